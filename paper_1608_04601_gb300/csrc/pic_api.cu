@@ -430,7 +430,10 @@ extern "C" pic_status pic_batch_create(pic_ctx** out, const pic_gas* gases, int3
                     v[(size_t)k] = d.V_rf_V * std::sin(2.0 * H_PI * d.f_rf_Hz * ((double)k * d.dt_s));
                 double* dv = nullptr;
                 ALLOC(dv, double*, sizeof(double) * (size_t)spp);
-                if (cudaMemcpy(dv, v.data(), sizeof(double) * (size_t)spp, cudaMemcpyHostToDevice) != cudaSuccess) {
+                // on the context's stream, behind the memset that clears the allocation (a copy on the
+                // legacy stream is not ordered with it and could be cleared after it landed)
+                if (cudaMemcpyAsync(dv, v.data(), sizeof(double) * (size_t)spp, cudaMemcpyHostToDevice,
+                                    ctx->stream) != cudaSuccess) {
                     pic_status s_ = fail(ctx, PIC_ERR_CUDA, "voltage table");
                     pic_destroy(ctx);
                     return s_;
@@ -445,8 +448,8 @@ extern "C" pic_status pic_batch_create(pic_ctx** out, const pic_gas* gases, int3
                 }
                 double* dj = nullptr;
                 ALLOC(dj, double*, sizeof(double) * 2 * (size_t)spp);
-                if (cudaMemcpy(dj, jt.data(), sizeof(double) * 2 * (size_t)spp, cudaMemcpyHostToDevice) !=
-                    cudaSuccess) {
+                if (cudaMemcpyAsync(dj, jt.data(), sizeof(double) * 2 * (size_t)spp, cudaMemcpyHostToDevice,
+                                    ctx->stream) != cudaSuccess) {
                     pic_status s_ = fail(ctx, PIC_ERR_CUDA, "current table");
                     pic_destroy(ctx);
                     return s_;
@@ -501,11 +504,6 @@ extern "C" pic_status pic_batch_create(pic_ctx** out, const pic_gas* gases, int3
             ctx->max_slices = std::max(ctx->max_slices, (int)ns);
             D.slice_n[sp] = (int)ns;
             ALLOC(D.slice_tot[sp], unsigned*, sizeof(unsigned) * 2 * 3 * ns);  // two parities
-            if (cudaMemset(D.slice_tot[sp], 0, sizeof(unsigned) * 2 * 3 * ns) != cudaSuccess) {
-                pic_status s_ = fail(ctx, PIC_ERR_CUDA, "slice sums");
-                pic_destroy(ctx);
-                return s_;
-            }
             if (sp == 0) {
                 ALLOC(D.sc, int32_t*, sizeof(int32_t) * (nrec + 16));
                 ALLOC(D.sp_, void*, rec * (nrec + 16));
@@ -822,6 +820,12 @@ extern "C" pic_status pic_sync(pic_ctx* ctx) {
 }
 
 // ---------------------------------------------------------------------------
+// Host -> device copy ordered with the context's stream, finished on return.
+static cudaError_t upload(pic_ctx* ctx, void* dst, const void* src, size_t bytes) {
+    cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, ctx->stream);
+    return e == cudaSuccess ? cudaStreamSynchronize(ctx->stream) : e;
+}
+
 static bool bad_d(pic_ctx* ctx, int d) { return !ctx || d < 0 || d >= ctx->n_disc; }
 
 // Pinned host scratch of at least `bytes` for read-backs: device -> host copies into it are
@@ -995,7 +999,7 @@ extern "C" pic_status pic_set_field(pic_ctx* ctx, int32_t d, const void* E) {
     if (bad_d(ctx, d) || !E) return PIC_ERR_ARG;
     CK(cudaStreamSynchronize(ctx->stream), "synchronize");
     const Disc& D = ctx->hd[d];
-    CK(cudaMemcpy(D.E, E, (ctx->fp64 ? 8 : 4) * ((size_t)D.N + 1), cudaMemcpyHostToDevice), "field");
+    CK(upload(ctx, D.E, E, (ctx->fp64 ? 8 : 4) * ((size_t)D.N + 1)), "field");
     return PIC_OK;
 }
 
@@ -1011,7 +1015,7 @@ extern "C" pic_status pic_set_deposit(pic_ctx* ctx, int32_t d, int32_t sp, const
     if (bad_d(ctx, d) || (sp & ~1) || !Dh) return PIC_ERR_ARG;
     CK(cudaStreamSynchronize(ctx->stream), "synchronize");
     const Disc& D = ctx->hd[d];
-    CK(cudaMemcpy(D.D[sp], Dh, 8 * ((size_t)D.N + 1), cudaMemcpyHostToDevice), "deposit");
+    CK(upload(ctx, D.D[sp], Dh, 8 * ((size_t)D.N + 1)), "deposit");
     ctx->deposits_zero = false;
     return PIC_OK;
 }
@@ -1034,7 +1038,7 @@ extern "C" pic_status pic_set_step(pic_ctx* ctx, int64_t step) {
     if (!ctx || step < 0) return PIC_ERR_ARG;
     CK(cudaStreamSynchronize(ctx->stream), "synchronize");
     long long v = step;
-    CK(cudaMemcpy(&ctx->d_ctl->step, &v, 8, cudaMemcpyHostToDevice), "step");
+    CK(upload(ctx, &ctx->d_ctl->step, &v, 8), "step");
     ctx->step = step;
     return PIC_OK;
 }
@@ -1214,7 +1218,7 @@ extern "C" pic_status pic_set_current_drive(pic_ctx* ctx, int32_t d, double J0) 
     if (bad_d(ctx, d) || !(J0 >= 0.0) || !std::isfinite(J0)) return PIC_ERR_ARG;
     if (!ctx->hd[d].jtab) return fail(ctx, PIC_ERR_STATE, "the time step does not divide the rf period");
     CK(cudaStreamSynchronize(ctx->stream), "synchronize");
-    CK(cudaMemcpy(&ctx->d_ctl->J_drive[d], &J0, sizeof(double), cudaMemcpyHostToDevice), "current drive");
+    CK(upload(ctx, &ctx->d_ctl->J_drive[d], &J0, sizeof(double)), "current drive");
     return PIC_OK;
 }
 
@@ -1243,9 +1247,8 @@ extern "C" pic_status pic_reset_moments(pic_ctx* ctx) {
     for (int d = 0; d < ctx->n_disc; ++d) {
         const Disc& D = ctx->hd[d];
         const size_t b = 16 * ((size_t)D.N + 1);
-        CK(cudaMemset(D.acc_D[0], 0, 4 * b), "reset");  // the four accumulators, one block
-        long long z = 0;
-        CK(cudaMemcpy(&ctx->d_ctl->acc_steps[d], &z, 8, cudaMemcpyHostToDevice), "reset");
+        CK(cudaMemsetAsync(D.acc_D[0], 0, 4 * b, ctx->stream), "reset");  // the four accumulators, one block
+        CK(cudaMemsetAsync(&ctx->d_ctl->acc_steps[d], 0, 8, ctx->stream), "reset");
         pic_status s = read_counters(ctx, d, &ctx->cnt_at_reset[d]);
         if (s != PIC_OK) return s;
     }
@@ -1510,15 +1513,17 @@ extern "C" pic_status pic_load_profiles(pic_ctx* ctx, int32_t n_pts, const doubl
         warm_desc_fill(ctx->fp64, desc.data() + dsz * d, base, base + P * r, base + 2 * P * r, P,
                        (double)ctx->dis[d].n_cells / (double)(P - 1), K23);
     }
-    cudaError_t e = cudaMemcpy(dtab, host.data(), host.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(ddesc, desc.data(), desc.size(), cudaMemcpyHostToDevice);
-    for (int d = 0; d < nd && e == cudaSuccess; ++d)
-        e = cudaMemcpy(&ctx->d_ctl->count[d][0], &counts[2 * d], 16, cudaMemcpyHostToDevice);
+    // everything on the context's stream, ahead of the load kernels
+    const cudaStream_t st = ctx->stream;
+    cudaError_t e = cudaMemcpyAsync(dtab, host.data(), host.size(), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(ddesc, desc.data(), desc.size(), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess)  // count[d][species] of consecutive discharges
+        e = cudaMemcpyAsync(&ctx->d_ctl->count[0][0], counts.data(), 16 * (size_t)nd, cudaMemcpyHostToDevice, st);
     for (auto& D : ctx->hd) {
         const size_t b = 8 * ((size_t)D.N + 1);
-        if (e == cudaSuccess) e = cudaMemset(D.D[0], 0, b);
-        if (e == cudaSuccess) e = cudaMemset(D.D[1], 0, b);
-        if (e == cudaSuccess) e = cudaMemset(D.Q, 0, b);
+        if (e == cudaSuccess) e = cudaMemsetAsync(D.D[0], 0, b, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(D.D[1], 0, b, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(D.Q, 0, b, st);
     }
     const int gx = std::max(1, ctx->num_sms * 4);
     ctx->cur = 0;
