@@ -358,9 +358,12 @@ extern "C" pic_status pic_batch_create(pic_ctx** out, const pic_gas* gases, int3
     auto bcap_of = [&](int i) {
         return std::max(ctx->dis[i].weights.capacity_e, ctx->dis[i].weights.capacity_i) / 8 + 4096;
     };
+    // host sources of asynchronous copies, alive until the stream is synchronised below
+    std::vector<long long> hoff(2 * MAXD, 0), eoff(2 * MAXD, 0);
+    std::vector<std::vector<double>> host_tabs;
+    host_tabs.reserve(2 * (size_t)n_dis);
     // sort scratch: per store (cells x sort tiles) counts
     {
-        std::vector<long long> hoff(2 * MAXD, 0);
         long long acc = 0;
         const long long st = sort_tile_chunks((int)chunk);
         for (int i = 0; i < n_dis; ++i)
@@ -375,7 +378,6 @@ extern "C" pic_status pic_batch_create(pic_ctx** out, const pic_gas* gases, int3
         ALLOC(ctx->sort_hoff, long long*, sizeof(long long) * 2 * MAXD);
         cudaMemcpyAsync(ctx->sort_hoff, hoff.data(), sizeof(long long) * 2 * MAXD, cudaMemcpyHostToDevice,
                         ctx->stream);
-        std::vector<long long> eoff(2 * MAXD, 0);
         long long ea = 0;
         for (int i = 0; i < n_dis; ++i)
             for (int sp = 0; sp < 2; ++sp) {
@@ -425,7 +427,8 @@ extern "C" pic_status pic_batch_create(pic_ctx** out, const pic_gas* gases, int3
             // one rf period of V(t) when dt divides it (f dt steps_per_period = 1 to 1e-12)
             const int spp = d.weights.steps_per_period;
             if (spp > 0 && std::fabs(d.f_rf_Hz * d.dt_s * spp - 1.0) <= 1e-12) {
-                std::vector<double> v((size_t)spp);
+                host_tabs.emplace_back((size_t)spp);
+                std::vector<double>& v = host_tabs.back();
                 for (int k = 0; k < spp; ++k)
                     v[(size_t)k] = d.V_rf_V * std::sin(2.0 * H_PI * d.f_rf_Hz * ((double)k * d.dt_s));
                 double* dv = nullptr;
@@ -440,7 +443,8 @@ extern "C" pic_status pic_batch_create(pic_ctx** out, const pic_gas* gases, int3
                 }
                 D.V0tab = dv;
                 // sin and cos at the step midpoints (first harmonic of J(t))
-                std::vector<double> jt(2 * (size_t)spp);
+                host_tabs.emplace_back(2 * (size_t)spp);
+                std::vector<double>& jt = host_tabs.back();
                 for (int k = 0; k < spp; ++k) {
                     const double ph = 2.0 * H_PI * d.f_rf_Hz * (((double)k + 0.5) * d.dt_s);
                     jt[2 * (size_t)k] = std::sin(ph);
