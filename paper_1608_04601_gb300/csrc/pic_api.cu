@@ -53,7 +53,8 @@ struct pic_ctx {
     int cur = 0;
     long long step = 0;
     bool deposits_zero = true;
-    int sweep_grid = 0, num_sms = 0;
+    int dep_par = 0;  // host copy of Ctl::dep_par
+    int sweep_grid = 0, sweep_warps = 0, sweep_sets = 0, num_sms = 0;
     int max_slices = 0;  // slices of sweep chunks of the largest store
     void* stage = nullptr;  // device staging of state transfers
     size_t stage_bytes = 0;
@@ -189,6 +190,44 @@ static void fill_consts(Consts<T>& k, const pic_derived& o, const pic_discharge&
     k.gamma = (T)d.weights.gamma_see;
     k.sig0[0] = (T)o.sig_e0;
     k.sig0[1] = (T)o.sig_i0;
+}
+
+// The sweep's view of the two stores of a discharge (every other field of D is set).
+template <typename T>
+static void fill_seg(Seg<T>* seg, const Disc& D, const Consts<T>& k) {
+    for (int sp = 0; sp < 2; ++sp) {
+        Seg<T> S{};
+        S.k = k;
+        S.N = D.N;
+        S.n_pts = D.n_pts;
+        S.has_see = D.has_see;
+        S.n_exc = D.n_exc;
+        S.leapfrog = D.leapfrog;
+        S.thr = D.thr[sp];
+        S.did = D.discharge_id;
+        S.slice_stride = 3 * D.slice_n[sp];
+        for (int b = 0; b < 2; ++b) {
+            S.c[b] = D.c[b][sp];
+            S.p[b] = D.p[b][sp];
+        }
+        S.start = D.start[sp];
+        S.bc = D.bc[sp];
+        S.bp = D.bp[sp];
+        S.sc = D.sc;
+        S.sp_ = D.sp_;
+        S.Te = D.Te;
+        S.Ti = D.Ti;
+        S.E = D.E;
+        S.Dg = D.D[sp];
+        S.Dother = D.D[1 - sp];
+        S.Qg = D.Q;
+        S.cnt = D.cnt;
+        S.cnt_main = D.cnt_main[sp];
+        S.cnt_birth = D.cnt_birth[sp];
+        S.cnt_same = D.cnt_same;
+        S.slice_tot = D.slice_tot[sp];
+        seg[sp] = S;
+    }
 }
 
 // Region bookkeeping of a store of capacity cap (superparticles) with sweep chunks of `chunk` slots
@@ -504,7 +543,7 @@ extern "C" pic_status pic_batch_create(pic_ctx** out, const pic_gas* gases, int3
             ALLOC(D.start[sp], int*, sizeof(int) * (mc + 2));
             ALLOC(D.cnt_main[sp], int*, sizeof(int) * (mc + 1));
             ALLOC(D.cnt_birth[sp], int*, sizeof(int) * (mc + 1));
-            const size_t ns = (mc + SLICE - 1) / SLICE + 1;
+            const size_t ns = (mc + SLICE - 1) / SLICE;
             ctx->max_slices = std::max(ctx->max_slices, (int)ns);
             D.slice_n[sp] = (int)ns;
             ALLOC(D.slice_tot[sp], unsigned*, sizeof(unsigned) * 2 * 3 * ns);  // two parities
@@ -518,10 +557,9 @@ extern "C" pic_status pic_batch_create(pic_ctx** out, const pic_gas* gases, int3
         ALLOC(D.E, void*, rsz * N1);
         ALLOC(D.E64, double*, 8 * N1);
         ALLOC(D.phi, double*, 8 * N1);
-        ALLOC(D.D[0], unsigned long long*, 8 * N1);
-        ALLOC(D.D[1], unsigned long long*, 8 * N1);
+        ALLOC(D.D[0], unsigned long long*, 2 * 8 * N1);  // two parities
+        ALLOC(D.D[1], unsigned long long*, 2 * 8 * N1);
         ALLOC(D.Q, unsigned long long*, 8 * N1);
-        ALLOC(D.Dprev, unsigned long long*, 8 * N1);
         // the four exact accumulators in one block (read back by one copy)
         ALLOC(D.acc_D[0], unsigned __int128*, 4 * 16 * N1);
         D.acc_D[1] = D.acc_D[0] + N1;
@@ -529,6 +567,8 @@ extern "C" pic_status pic_batch_create(pic_ctx** out, const pic_gas* gases, int3
         D.acc_Dprev = D.acc_D[0] + 3 * N1;
         ALLOC(D.cnt, unsigned long long*, 8 * NCNT);
         ALLOC(D.period_mean, double*, sizeof(double) * 2 * PERIOD_HIST);
+        if (ctx->fp64) fill_seg<double>(D.sd, D, D.cd);
+        else fill_seg<float>(D.sf, D, D.cf);
         ctx->hd.push_back(D);
         std::memset(&ctx->cnt_at_reset[i], 0, sizeof(pic_counters));
     }
@@ -541,7 +581,7 @@ extern "C" pic_status pic_batch_create(pic_ctx** out, const pic_gas* gases, int3
         for (int i = 0; i < n_dis; ++i) {
             h.count[i][0] = o.load ? ctx->dis[i].weights.n_e0 : 0;
             h.count[i][1] = o.load ? ctx->dis[i].weights.n_i0 : 0;
-            h.V_scale[i] = 1.0;
+            h.V_scale[i][0] = h.V_scale[i][1] = 1.0;
             h.J_drive[i] = 0.0;
         }
         cudaMemcpyAsync(ctx->d_ctl, &h, sizeof(Ctl), cudaMemcpyHostToDevice, ctx->stream);
@@ -553,12 +593,14 @@ extern "C" pic_status pic_batch_create(pic_ctx** out, const pic_gas* gases, int3
             return s;
         }
     }
-    // sweep grid: persistent CTAs
+    // sweep grid: one persistent CTA per SM
     {
-        int occ = sweep_occupancy(ctx->fp64, o.block, o.ppt, ctx->max_N, n_dis);
-        if (occ < 1) occ = 1;
-        int per = o.ctas_per_sm > 0 ? std::min(o.ctas_per_sm, occ) : occ;
-        ctx->sweep_grid = std::max(1, ctx->num_sms * per);
+        ctx->sweep_grid = std::max(1, ctx->num_sms);
+        long long chunks = 0;
+        for (auto& D : ctx->hd) chunks += (D.cap[0] + chunk - 1) / chunk + (D.cap[1] + chunk - 1) / chunk;
+        const int want = o.ctas_per_sm > 0 ? std::min(o.block, 512) * std::min(o.ctas_per_sm, 16) / 32 : 0;
+        sweep_shape(ctx->fp64, o.ppt, ctx->max_N, n_dis, want, (chunks + ctx->sweep_grid - 1) / ctx->sweep_grid,
+                    &ctx->sweep_warps, &ctx->sweep_sets);
     }
     if (o.load) {
         const int gx = std::max(1, ctx->num_sms * 4);
@@ -576,6 +618,7 @@ extern "C" pic_status pic_batch_create(pic_ctx** out, const pic_gas* gases, int3
     }
     ctx->cur = 0;
     ctx->step = 0;
+    ctx->dep_par = o.load ? 1 : 0;  // the initial solve of a load flips it
     ctx->deposits_zero = true;
     // Sweeps append regions (one per chunk, plus the newborns' chunks); a sort makes a store dense
     // again. When it runs rarer than every 64 steps, an order-preserving repack does, every R steps
@@ -614,19 +657,27 @@ extern "C" pic_status pic_create(pic_ctx** out, const pic_gas* gas, double gap_m
 }
 
 // ---------------------------------------------------------------------------
-static pic_status enqueue_sweep(pic_ctx* ctx) {
-    if (!ctx->deposits_zero) {
-        for (auto& D : ctx->hd) {
-            const size_t b = 8 * ((size_t)D.N + 1);
-            CK(cudaMemsetAsync(D.D[0], 0, b, ctx->stream), "memset");
-            CK(cudaMemsetAsync(D.D[1], 0, b, ctx->stream), "memset");
-            CK(cudaMemsetAsync(D.Q, 0, b, ctx->stream), "memset");
-        }
+// The deposits the next sweep adds to, cleared if a sweep or an upload left something in them.
+static pic_status zero_deposits(pic_ctx* ctx) {
+    if (ctx->deposits_zero) return PIC_OK;
+    for (auto& D : ctx->hd) {
+        const size_t n1 = (size_t)D.N + 1, o = ctx->dep_par * n1;
+        CK(cudaMemsetAsync(D.D[0] + o, 0, 8 * n1, ctx->stream), "memset");
+        CK(cudaMemsetAsync(D.D[1] + o, 0, 8 * n1, ctx->stream), "memset");
+        CK(cudaMemsetAsync(D.Q, 0, 8 * n1, ctx->stream), "memset");
     }
+    ctx->deposits_zero = true;
+    return PIC_OK;
+}
+
+static pic_status enqueue_sweep(pic_ctx* ctx) {
+    pic_status sz = zero_deposits(ctx);
+    if (sz != PIC_OK) return sz;
     SweepLaunch L{};
     L.fp64 = ctx->fp64;
-    L.block = ctx->opt.block;
     L.ppt = ctx->opt.ppt;
+    L.warps = ctx->sweep_warps;
+    L.sets = ctx->sweep_sets;
     L.grid = ctx->sweep_grid;
     L.max_N = ctx->max_N;
     L.n_disc = ctx->n_disc;
@@ -658,6 +709,7 @@ static pic_status enqueue_finalize(pic_ctx* ctx, int mode) {
        "finalize launch");
     if (mode & 1) ctx->cur = 1 - ctx->cur;
     if (mode & 2) ctx->step += 1;
+    ctx->dep_par ^= 1;
     ctx->deposits_zero = true;
     return PIC_OK;
 }
@@ -731,6 +783,10 @@ static pic_status enqueue_step(pic_ctx* ctx) {
 }
 
 static pic_status run_graph_period(pic_ctx* ctx, int P) {
+    // deposits left by a single sweep or an upload are cleared outside the graph (their parity differs
+    // from one launch to the next if the period has an odd number of steps)
+    pic_status sz = zero_deposits(ctx);
+    if (sz != PIC_OK) return sz;
     // the period's sorts and repacks follow from the step at which it starts
     const int phase = (int)(ctx->step % P);
     for (auto& g : ctx->graphs)
@@ -738,11 +794,11 @@ static pic_status run_graph_period(pic_ctx* ctx, int P) {
             CK(cudaGraphLaunch(g.exec, ctx->stream), "graph launch");
             ctx->cur = g.cur_out;
             ctx->step += P;
-            ctx->deposits_zero = true;
+            ctx->dep_par ^= P & 1;
             return PIC_OK;
         }
     // capture one period
-    const int cur0 = ctx->cur;
+    const int cur0 = ctx->cur, dep0 = ctx->dep_par;
     const long long step0 = ctx->step;
     const bool timing = ctx->timing;
     ctx->timing = false;
@@ -752,6 +808,7 @@ static pic_status run_graph_period(pic_ctx* ctx, int P) {
     for (int i = 0; i < P && s == PIC_OK; ++i) s = enqueue_step(ctx);
     cudaError_t e = cudaStreamEndCapture(ctx->stream, &graph);
     ctx->timing = timing;
+    ctx->dep_par = dep0;
     if (s != PIC_OK) return s;
     if (e != cudaSuccess) return cuda_fail(ctx, e, "end capture");
     cudaGraphExec_t exec;
@@ -765,7 +822,7 @@ static pic_status run_graph_period(pic_ctx* ctx, int P) {
     CK(cudaGraphLaunch(exec, ctx->stream), "graph launch");
     ctx->cur = ge.cur_out;
     ctx->step = step0 + P;
-    ctx->deposits_zero = true;
+    ctx->dep_par = dep0 ^ (P & 1);
     return PIC_OK;
 }
 
@@ -1011,7 +1068,8 @@ extern "C" pic_status pic_get_deposit(pic_ctx* ctx, int32_t d, int32_t sp, int64
     if (bad_d(ctx, d) || (sp & ~1) || !Dh) return PIC_ERR_ARG;
     CK(cudaStreamSynchronize(ctx->stream), "synchronize");
     const Disc& D = ctx->hd[d];
-    CK(cudaMemcpy(Dh, D.D[sp], 8 * ((size_t)D.N + 1), cudaMemcpyDeviceToHost), "deposit");
+    const size_t n1 = (size_t)D.N + 1;
+    CK(cudaMemcpy(Dh, D.D[sp] + ctx->dep_par * n1, 8 * n1, cudaMemcpyDeviceToHost), "deposit");
     return PIC_OK;
 }
 
@@ -1019,7 +1077,8 @@ extern "C" pic_status pic_set_deposit(pic_ctx* ctx, int32_t d, int32_t sp, const
     if (bad_d(ctx, d) || (sp & ~1) || !Dh) return PIC_ERR_ARG;
     CK(cudaStreamSynchronize(ctx->stream), "synchronize");
     const Disc& D = ctx->hd[d];
-    CK(upload(ctx, D.D[sp], Dh, 8 * ((size_t)D.N + 1)), "deposit");
+    const size_t n1 = (size_t)D.N + 1;
+    CK(upload(ctx, D.D[sp] + ctx->dep_par * n1, Dh, 8 * n1), "deposit");
     ctx->deposits_zero = false;
     return PIC_OK;
 }
@@ -1236,7 +1295,7 @@ extern "C" pic_status pic_voltage_amplitude(pic_ctx* ctx, int32_t d, int64_t fir
     if (periods_done) *periods_done = done;
     if (V0_now) {
         double s = 1.0;
-        CK(cudaMemcpy(&s, &ctx->d_ctl->V_scale[d], sizeof(double), cudaMemcpyDeviceToHost), "voltage");
+        CK(cudaMemcpy(&s, &ctx->d_ctl->V_scale[d][ctx->dep_par], sizeof(double), cudaMemcpyDeviceToHost), "voltage");
         *V0_now = D.V_rf * s;
     }
     if (!D.jtab && n > 0) return fail(ctx, PIC_ERR_STATE, "the time step does not divide the rf period");
@@ -1525,8 +1584,8 @@ extern "C" pic_status pic_load_profiles(pic_ctx* ctx, int32_t n_pts, const doubl
         e = cudaMemcpyAsync(&ctx->d_ctl->count[0][0], counts.data(), 16 * (size_t)nd, cudaMemcpyHostToDevice, st);
     for (auto& D : ctx->hd) {
         const size_t b = 8 * ((size_t)D.N + 1);
-        if (e == cudaSuccess) e = cudaMemsetAsync(D.D[0], 0, b, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(D.D[1], 0, b, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(D.D[0], 0, 2 * b, st);  // both parities
+        if (e == cudaSuccess) e = cudaMemsetAsync(D.D[1], 0, 2 * b, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(D.Q, 0, b, st);
     }
     const int gx = std::max(1, ctx->num_sms * 4);
@@ -1541,6 +1600,7 @@ extern "C" pic_status pic_load_profiles(pic_ctx* ctx, int32_t n_pts, const doubl
     cudaFree(dtab);
     cudaFree(ddesc);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "warm start");
+    ctx->dep_par ^= 1;  // the solve
     ctx->deposits_zero = true;
     return PIC_OK;
 }

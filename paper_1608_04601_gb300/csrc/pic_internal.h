@@ -60,6 +60,34 @@ struct Lay {
     long long D0;             // record offset of the dense part
 };
 
+// One store of a discharge (a species) as the sweep uses it, prepared by the host so that a CTA fetches
+// it in one coalesced copy into shared memory. Arrays [2] of buffers by record buffer.
+template <typename T>
+struct Seg {
+    Consts<T> k;
+    int N, n_pts, has_see, n_exc, leapfrog;
+    uint32_t thr, did;
+    int slice_stride;         // slice sums of one parity
+    int32_t* c[2];            // the store's records
+    void* p[2];
+    const int* start;
+    int32_t* bc;              // other-species newborns of this sweep, chunk regions
+    void* bp;
+    int32_t* sc;              // same-species newborns (ionization electrons), chunk regions
+    void* sp_;
+    const void* Te;
+    const void* Ti;
+    const void* E;
+    unsigned long long* Dg;   // deposits of this species and of the other one, parity 0
+    unsigned long long* Dother;
+    unsigned long long* Qg;
+    unsigned long long* cnt;
+    int* cnt_main;
+    int* cnt_birth;
+    int* cnt_same;
+    unsigned* slice_tot;      // parity 0
+};
+
 struct Disc {
     int N, n_exc, n_pts, gas;
     uint32_t thr[2];          // null-collision candidate thresholds (of 2^32)
@@ -104,9 +132,11 @@ struct Disc {
     void* E;                  // node field for the gather (T), N+1
     double* E64;              // node field, FP64
     double* phi;              // potential, FP64
-    unsigned long long* D[2]; // CIC deposits at x_{n+1}, 2^32 per particle
+    // CIC deposits, 2^32 per particle: two arrays of N+1 by parity. The sweep adds the deposit at x_{n+1}
+    // to the array of Ctl::dep_par; the solve reads it, takes the other one as the deposit at x_n, clears
+    // that for the next sweep and flips the parity
+    unsigned long long* D[2];
     unsigned long long* Q;    // electron energy moment at x_n, 2^-12 eV
-    unsigned long long* Dprev;// electron deposit at x_n
     unsigned __int128* acc_D[2];    // exact sums over the accumulated steps of D, Q, D at x_n
     unsigned __int128* acc_Q;
     unsigned __int128* acc_Dprev;
@@ -125,6 +155,8 @@ struct Disc {
     double* dg_E;
     unsigned long long* dg_eedf;
     unsigned long long* dg_n;
+    Seg<float> sf[2];         // [species], filled in the context's precision only
+    Seg<double> sd[2];
 };
 
 // Node arrays of the kinetic diagnostics (k_diag): density, energy, particle flux, energy flux,
@@ -156,6 +188,7 @@ struct Ctl {
     Lay lay[MAXD][2][2];      // [discharge][species][buffer] layout of the store in that buffer
     int chunks_in[MAXD][2];   // chunks the last sweep processed, per store
     int slice_par;            // parity of the slice sums the next sweep adds into
+    int dep_par;              // parity of the deposits the next sweep adds into
     long long acc_steps[MAXD];
     double E0_last[MAXD];
     // J(t): electrode fields and event counters at the last solve, first-harmonic sums of the
@@ -165,8 +198,9 @@ struct Ctl {
     unsigned long long cnt_solve[MAXD][6];
     double J_sum[MAXD][2];
     // current-driven mode (Eq. adaptivevoltage): the applied amplitude is V_rf V_scale, and with
-    // J_drive > 0 V_scale <- V_scale J_drive / J_calc after every rf period
-    double V_scale[MAXD];
+    // J_drive > 0 V_scale <- V_scale J_drive / J_calc after every rf period; a solve reads the one of
+    // dep_par and writes the other
+    double V_scale[MAXD][2];
     double J_drive[MAXD];
     double period_acc[MAXD][2];   // sum of the counts over the steps of the current rf period
     unsigned sort_rows_done[MAXD][2];  // k_sort_rows CTAs finished, per store (reset by the last)

@@ -2,15 +2,15 @@
 // arXiv:1608.04601, section "PIC/MCC simulation procedure".
 //
 // One time step is two launches (and the sort every K steps):
-//   k_sweep     persistent; tiles of BLOCK x PPT slots of all stores in a
-//               static grid-stride order; each warp owns a chunk of 32 PPT
-//               slots and loads, pushes (CIC gather of E_n from shared
-//               memory, half kick, null-collision MCC on Philox streams, half
-//               kick, drift, walls), collides and writes its survivors in slot
-//               order into the chunk's own output region, newborns into the
-//               chunk's newborn regions, with no barrier inside a tile. CIC
-//               deposits go to warp-aggregated shared-memory int64 histograms,
-//               flushed with global atomics. Chunk counts are summed per slice.
+//   k_sweep     persistent, one CTA per SM; every warp takes a contiguous run
+//               of chunks (32 PPT slots) of each store and per chunk draws the
+//               candidates, collides them, then pushes all its particles in one
+//               pass (CIC gather of E_n from shared memory, half kicks, drift,
+//               walls) and writes the survivors in slot order into the chunk's
+//               own output region, newborns into the chunk's newborn regions.
+//               CIC deposits and energy go to shared-memory histograms of exact
+//               32-bit pieces, flushed with global atomics. Chunk counts are
+//               summed per slice.
 //   k_post      per slice of chunks: the region starts of the new layout and
 //               the newborn copies; per discharge, concurrently: the store
 //               totals (new counts) and Poisson (Eq. poisson, rf Dirichlet
@@ -42,52 +42,23 @@ template <> struct T4<float> { using type = float4; using two = float2; };
 template <> struct T4<double> { using type = d4; using two = double2; };
 
 template <int V>
-struct IC {
-    static constexpr int value = V;
-};
-
+struct IC { static constexpr int value = V; };
 template <typename T>
 struct Part {
     int c;
     T f, vx, vy, vz;
 };
 
-// Segment (one store of one discharge) as seen by a sweep CTA.
-template <typename T>
-struct Seg {
-    Consts<T> k;
-    int d, sp, N, n_pts, has_see, n_exc, leapfrog;
-    uint32_t thr, did;
-    long long n, cap, bcap, tile0, ntiles;
-    const int32_t* cin;
-    const void* pin;
-    int32_t* cout;
-    void* pout;
-    int32_t* bc;      // other-species newborns of this sweep, chunk regions
-    void* bp;
-    int32_t* sc;      // same-species newborns (ionization electrons), chunk regions
-    void* sp_;
-    const void* Te;
-    const void* Ti;
-    unsigned long long* Dg;
-    unsigned long long* Dother;
-    unsigned long long* Qg;
-    unsigned long long* cnt;
-    const int* start;  // region starts of the input layout
-    int K;             // region chunks of the input layout
-    long long M, D0;   // slots in the regions, record offset of the dense part
-    long long ralloc;  // output regions
-    int* cnt_main;
-    int* cnt_birth;
-    int* cnt_same;
-    unsigned* slice_tot;
-};
+template <typename T> __device__ __forceinline__ const Seg<T>* segs_of(const Disc& d);
+template <> __device__ __forceinline__ const Seg<float>* segs_of<float>(const Disc& d) { return d.sf; }
+template <> __device__ __forceinline__ const Seg<double>* segs_of<double>(const Disc& d) { return d.sd; }
 
 // Programmatic dependent launch (the kernels of a step, launched by launch_pdl): wait until the
-// previous kernel in the stream has completed and its writes are visible. Every such kernel calls
-// this before its first memory access (a no-op for a kernel launched without the attribute). No
-// kernel triggers its dependents early: they launch as its CTAs exit, so no CTA of a later kernel
-// shares an SM's L1 with a CTA that may still read data the kernel in between rewrites.
+// previous kernel in the stream has completed and its writes are visible. Every such kernel calls this
+// before its first access to memory that kernels write (a no-op for a kernel launched without the
+// attribute); what needs no results (shared memory cleared, constants fetched) may come before. No kernel
+// triggers its dependents early: they launch as its CTAs exit (with early triggers in the sweep and k_post
+// the smallest runs gained 0.6 us of 26 a step and the larger ones lost 1-2 %).
 __device__ __forceinline__ void grid_dep_sync() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename T>
@@ -102,6 +73,27 @@ __device__ __forceinline__ int drift(int N, T dtdx, int c, T f, T vz, int& cn, T
     cn = c + (int)fl;
     fn = fr;
     return -1;
+}
+
+// The drift of the sweep's main pass, the same values as drift() with fewer operations: floor(s) by
+// adding 1.5 2^23 (2^52 in double) rounded towards minus infinity, which leaves the integer in the low
+// mantissa bits; exact for |s| < 8192, and a particle further out (or not a number) is not alive: a
+// discharge has at most 4096 cells. Returns whether the particle stays; s >= 0 then tells the electrode.
+__device__ __forceinline__ bool drift_fast(int N, float dtdx, int c, float f, float vz, int& cn, float& fn, float& s) {
+    s = __fmaf_rn(vz, dtdx, f);
+    const float t = __fadd_rd(s, 12582912.0f);
+    cn = c + (__float_as_int(t) - 0x4B400000);
+    fn = fminf(__fsub_rn(s, __fsub_rn(t, 12582912.0f)), one_minus_ulp<float>());
+    return fabsf(s) < 8192.0f && (unsigned)cn < (unsigned)N;
+}
+__device__ __forceinline__ bool drift_fast(int N, double dtdx, int c, double f, double vz, int& cn, double& fn,
+                                           double& s) {
+    s = __fma_rn(vz, dtdx, f);
+    const double t = __dadd_rd(s, 6755399441055744.0);
+    cn = c + __double2loint(t);
+    fn = __dsub_rn(s, __dsub_rn(t, 6755399441055744.0));
+    if (__double2hiint(fn) >= 0x3FF00000) fn = one_minus_ulp<double>();  // rounded to 1
+    return (__double2hiint(s) & 0x7FFFFFFF) < 0x40C00000 && (unsigned)cn < (unsigned)N;  // |s| < 8192
 }
 
 // Exact 64-bit add into a shared-memory word with native 32-bit atomics: the low
@@ -126,84 +118,98 @@ __device__ __forceinline__ void shist_add(unsigned long long* h, int c, unsigned
 }
 
 // Round-to-nearest-even conversion of a value in [0, 2^32) to an unsigned integer.
-__device__ __forceinline__ unsigned long long rint_u32(float a) { return __float2uint_rn(a); }
-__device__ __forceinline__ unsigned long long rint_u32(double a) { return __double2uint_rn(a); }
+__device__ __forceinline__ unsigned rint_u32(float a) { return __float2uint_rn(a); }
+__device__ __forceinline__ unsigned rint_u32(double a) {
+    return (unsigned)__double2loint(__dadd_rn(a, 6755399441055744.0));  // 1.5 2^52: the integer in the low bits
+}
 
 __device__ __forceinline__ unsigned long long cic_F(float f) {
     return (unsigned long long)__float2uint_rn(__fmul_rn(f, 4294967296.0f));  // f < 1: below 2^32
 }
+// May round to 2^32. Adding 1.5 2^20 rounds f to a multiple of 2^-32 (ties to even) and leaves the
+// multiple in the low mantissa bits: one FP64 addition (the FP64 pipe is the slow one here).
 __device__ __forceinline__ unsigned long long cic_F(double f) {
-    return __double2ull_rn(__dmul_rn(f, TWO32_D));  // may round to 2^32
+    return (unsigned long long)(__double_as_longlong(__dadd_rn(f, 1572864.0)) - 0x4138000000000000ll);
 }
-
-// Warp-aggregated histogram updates (warp_dep, warp_energy below; k_diag): lanes with equal keys are
-// grouped (match_any) and each group's sums reduced (redux) and added by its first lane. The group
-// reductions of a warp run one after another (one per distinct member mask), so their cost grows
-// with the number of groups: a warp with more than HIST_GROUPS distinct keys adds lane by lane
-// instead (measured on C2 with the earlier 64-bit adds: the sweep of an unsorted store 140 -> 55
-// us; two groups was the best threshold within a sort period). Integer adds: the same sums either way.
-constexpr int HIST_GROUPS = 2;
 
 // The sweep's shared-memory histograms hold exact sums in 32-bit pieces, added with atomics whose
-// result is not read (no return trip, no carry logic):
-//   deposit, per cell c: particles n_c, and the sum of F = rn(f 2^32) as low and high 16-bit parts;
-//     node j then receives 2^32 n_j - F_j + F_{j-1} (the charge split (2^32 - F, F) of every
-//     particle), formed in 64 bits when the CTA flushes;
-//   energy moment, per node: the sum of its 26-bit values as low 13-bit and high parts.
-// A piece sum stays below 2^32 while the CTA has added fewer than 2^15 particles (plus their
-// newborns) since its last flush: the sweep flushes at least that often.
-struct DepHist {
-    unsigned* n;
-    unsigned* lo;
-    unsigned* hi;
+// result is not read (no return trip, no carry logic); arrays of one word per cell c, `hs` words apart:
+//   0 particles n_c; 1, 2 the sum of F = rn(f 2^32) as low and high 16-bit parts; node j then receives
+//     2^32 n_j - F_j + F_{j-1} (the charge split (2^32 - F, F) of every particle);
+//   3, 4 (electrons) the sums of the low 17 bits of the energy E and of its share H = rn(E f); node j
+//     receives E_j - H_j + H_{j-1}. The bits above (an electron of more than 32 eV) go straight to the
+//     global sums.
+// The 64-bit node values are formed when the CTA flushes. A piece sum stays below 2^32 while the CTA has
+// added at most FLUSH_PARTICLES particles of a species (plus as many newborns) since its last flush.
+template <typename T>
+__host__ __device__ constexpr int flush_particles() { return sizeof(T) == 4 ? 32768 : 16384; }  // F = 2^32 occurs in double
+//
+// On a cell-sorted store the lanes of a warp add to the same few cells, and adds to one word run one
+// after another. So each species also has a window of WIN cells around the CTA's chunks with WCOP copies
+// of every word, lane l adding to copy l % WCOP: at most 32 / WCOP adds meet. A flush folds the window
+// into the full arrays. (The sweep of a freshly sorted store of 1.2e7 + 1.2e7 particles in 2048 cells
+// spent a third of its time in these conflicts.)
+// A CTA with fewer than WIN_CHUNKS chunks of a store goes without: it has few adds, and the extra pass of
+// its flush costs more (2e4 + 2e4 particles: 22.4 us a step with windows everywhere, 21.5 with this rule).
+constexpr int WIN = 64, WCOP = 8, WWORDS = WIN * WCOP, WIN_CHUNKS = 16, NO_WIN = -(1 << 30);
+struct Hist {
+    unsigned* full;  // arrays of hs words
+    unsigned* win;   // arrays of WWORDS words: cell w0 + j, copy k at j WCOP + k
+    int hs, w0;
+    // the words of cell c for this lane: first array and distance between arrays
+    __device__ __forceinline__ unsigned* at(int c, int lane, int& st) const {
+        const unsigned j = (unsigned)(c - w0);
+        const bool in = j < (unsigned)WIN;
+        st = in ? WWORDS : hs;
+        return in ? win + (j * WCOP + (lane & (WCOP - 1))) : full + c;
+    }
 };
-__device__ __forceinline__ void dep_add(const DepHist& h, int c, unsigned long long F) {
-    atomicAdd(&h.n[c], 1u);
-    atomicAdd(&h.lo[c], (unsigned)(F & 0xFFFFu));
-    atomicAdd(&h.hi[c], (unsigned)(F >> 16));
+__device__ __forceinline__ void dep_add(const Hist& h, int c, unsigned long long F, int lane) {
+    int st;
+    unsigned* a = h.at(c, lane, st);
+    atomicAdd(a, 1u);
+    atomicAdd(a + st, (unsigned)(F & 0xFFFFu));
+    atomicAdd(a + 2 * st, (unsigned)(F >> 16));
 }
-// Warp-aggregated deposit of one particle per lane (key = cell, < 0: none; F as above): lanes of
-// equal keys are reduced (match_any, redux) and their first lane adds the group's sums, unless the
-// warp's keys form more than HIST_GROUPS groups (then lane by lane).
-__device__ __forceinline__ void warp_dep(const DepHist& h, int key, unsigned long long F, int lane) {
-    const int k0 = __shfl_sync(FULL, key, 0);
-    if (!__all_sync(FULL, key == k0)) {  // several cells (or empty lanes): lane by lane
-        if (key >= 0) dep_add(h, key, F);
-        return;
-    }
-    const unsigned lo = __reduce_add_sync(FULL, (unsigned)(F & 0xFFFFu));
-    const unsigned hi = __reduce_add_sync(FULL, (unsigned)(F >> 16));
-    if (lane == 0 && key >= 0) {
-        atomicAdd(&h.n[key], 32u);
-        if (lo) atomicAdd(&h.lo[key], lo);
-        if (hi) atomicAdd(&h.hi[key], hi);
-    }
-}
-// Warp-aggregated energy moment: a (< 2^26) to node key, b (< 2^26) to node key + 1.
-__device__ __forceinline__ void warp_energy(unsigned* qlo, unsigned* qhi, int key, unsigned a, unsigned b, int lane) {
-    const int k0 = __shfl_sync(FULL, key, 0);
-    const unsigned peers = FULL;
-    const bool leader = lane == 0;
-    if (!__all_sync(FULL, key == k0)) {
-        if (key >= 0) {
-            if (a) {
-                atomicAdd(&qlo[key], a & 0x1FFFu);
-                atomicAdd(&qhi[key], a >> 13);
+// Deposit of one particle per lane (key = cell, < 0: none). UNIFORM (ions: slow, so a row of a sorted
+// store mostly shares a cell): such a row is reduced across the warp and added by one lane.
+template <bool UNIFORM>
+__device__ __forceinline__ void warp_dep(const Hist& h, int key, unsigned long long F, int lane) {
+    if (UNIFORM) {
+        const int k0 = __shfl_sync(FULL, key, 0);
+        if (__all_sync(FULL, key == k0)) {
+            const unsigned lo = __reduce_add_sync(FULL, (unsigned)(F & 0xFFFFu));
+            const unsigned hi = __reduce_add_sync(FULL, (unsigned)(F >> 16));
+            if (lane == 0 && key >= 0) {
+                int st;
+                unsigned* a = h.at(key, lane, st);
+                atomicAdd(a, 32u);
+                atomicAdd(a + st, lo);
+                atomicAdd(a + 2 * st, hi);
             }
-            if (b) {
-                atomicAdd(&qlo[key + 1], b & 0x1FFFu);
-                atomicAdd(&qhi[key + 1], b >> 13);
-            }
+            return;
         }
-        return;
     }
-    const unsigned al = __reduce_add_sync(peers, a & 0x1FFFu), ah = __reduce_add_sync(peers, a >> 13);
-    const unsigned bl = __reduce_add_sync(peers, b & 0x1FFFu), bh = __reduce_add_sync(peers, b >> 13);
-    if (leader && key >= 0) {
-        if (al) atomicAdd(&qlo[key], al);
-        if (ah) atomicAdd(&qhi[key], ah);
-        if (bl) atomicAdd(&qlo[key + 1], bl);
-        if (bh) atomicAdd(&qhi[key + 1], bh);
+    if (key >= 0) dep_add(h, key, F, lane);
+}
+// Energy moment of the lanes' electrons (`on`; every lane of the warp calls) of energy speed^2 kappa_E
+// (2^-12 eV, clamped at 2^26) at (c, f).
+template <typename T>
+__device__ __forceinline__ void energy_add(const Hist& h, unsigned long long* Qg, bool on, int c, T f, T e2, T kappa_E,
+                                           int lane) {
+    T eq = mul_(e2, kappa_E);
+    if (!(eq <= (T)0x1p26)) eq = (T)0x1p26;
+    const unsigned Et = rint_u32(eq), Eh = rint_u32(mul_(eq, f));
+    if (on) {
+        int st;
+        unsigned* a = h.at(c, lane, st);
+        atomicAdd(a + 3 * st, Et & 0x1FFFFu);
+        atomicAdd(a + 4 * st, Eh & 0x1FFFFu);
+    }
+    if (__any_sync(FULL, on && (Et >> 17)) && on && (Et >> 17)) {
+        const unsigned long long ht = Et >> 17, hh = Eh >> 17;
+        atomicAdd(&Qg[c], (ht - hh) << 17);
+        if (hh) atomicAdd(&Qg[c + 1], hh << 17);
     }
 }
 
@@ -238,6 +244,44 @@ __device__ __forceinline__ void load_rec<double>(const void* p, unsigned i, doub
     f = a.x; vx = a.y; vy = b.x; vz = b.y;
 }
 
+// The random draws, directions and normals of a collision out of line: they appear several times in
+// the sweep, and its instructions are what a short sweep waits for.
+__device__ __forceinline__ U4 draw_call(unsigned long long seed, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3) {
+    return philox4x32_10(c0, c1, c2, c3, (uint32_t)seed, (uint32_t)(seed >> 32));
+}
+__device__ __forceinline__ float3 iso_dir_call(float ua, float ub) {
+    float3 n;
+    iso_dir(ua, ub, n.x, n.y, n.z);
+    return n;
+}
+__device__ __forceinline__ float2 box_muller_call(float ua, float ub) {
+    float2 n;
+    box_muller(ua, ub, n.x, n.y);
+    return n;
+}
+__device__ __forceinline__ void direction(float ua, float ub, float& x, float& y, float& z) {
+    const float3 n = iso_dir_call(ua, ub);
+    x = n.x;
+    y = n.y;
+    z = n.z;
+}
+__device__ __forceinline__ void direction(float ua, float ub, double& x, double& y, double& z) {
+    iso_dir(ua, ub, x, y, z);
+}
+__device__ __forceinline__ void normals(float ua, float ub, float& a, float& b) {
+    const float2 n = box_muller_call(ua, ub);
+    a = n.x;
+    b = n.y;
+}
+// draw() of pic_device.cuh with the counter's second and third words prepared once.
+struct Stream {
+    unsigned long long seed;
+    uint32_t w1, w2, did;  // step bits 0..31; step bits 32..47 << 16 | species << 8; discharge
+    __device__ __forceinline__ U4 draw(uint32_t slot, int call) const {
+        return draw_call(seed, slot, w1, w2 | (uint32_t)call, did);
+    }
+};
+
 // The collision candidates of a chunk are queued by their warp in shared memory as their indices
 // in the chunk; the lane that processes one reads the particle from the staged records, collides
 // it, writes the new velocity back into the staged record and flags the newborns it left after
@@ -254,8 +298,8 @@ struct Cand {
 // The collision of a queued candidate (null-collision method: process
 // selection against the cumulative rate tables, then the kinematics).
 template <typename T>
-__device__ __forceinline__ uint32_t collide(const Seg<T>& S, Cand<T>& q, int qc, T qf, uint32_t slot, uint32_t ridx,
-                                         long long step, unsigned long long seed, const DepHist& sH, unsigned* sC,
+__device__ __forceinline__ uint32_t collide(const Seg<T>& S, int SP, unsigned long long* Dother, Cand<T>& q, int qc, T qf, uint32_t slot, uint32_t ridx,
+                                         const Stream& rs, const Hist& sH, unsigned* sC,
                                          int& err) {
     using Row4 = typename T4<T>::type;
     using Row2 = typename T4<T>::two;
@@ -263,26 +307,23 @@ __device__ __forceinline__ uint32_t collide(const Seg<T>& S, Cand<T>& q, int qc,
     const int N = S.N;
     T vx = q.vx, vy = q.vy, vz = q.vz;
     uint32_t out = 0;
-    if (S.sp == 0) {
+    if (SP == 0) {
         const T e2 = fma_(vx, vx, fma_(vy, vy, mul_(vz, vz)));
         bool child = false;
         T cvx = 0, cvy = 0, cvz = 0, ivx = 0, ivy = 0, ivz = 0;
-        const U4 r = draw(seed, slot, step, 0, 0, S.did);
+        // the two table rows are requested first, so that their latency runs under the draw
         const T xi = mul_(e2, K.kappa_e);
-        const Row4* Te = reinterpret_cast<const Row4*>(S.Te);
-        T C0, C1, C2, C3;
-        if (!(xi < (T)(S.n_pts - 1))) {
-            const Row4 a = Te[S.n_pts - 1];
-            C0 = a.x; C1 = a.y; C2 = a.z; C3 = a.w;
+        const bool above = !(xi < (T)(S.n_pts - 1));  // beyond the last row: its values
+        const int it = above ? S.n_pts - 2 : (int)xi;
+        const Row4* Te = reinterpret_cast<const Row4*>(S.Te) + it;
+        const Row4 ta = Te[0], tb = Te[1];
+        const U4 r = rs.draw(slot, 0);
+        const T fr = sub_(xi, (T)it);
+        T C0 = fma_(fr, sub_(tb.x, ta.x), ta.x), C1 = fma_(fr, sub_(tb.y, ta.y), ta.y);
+        T C2 = fma_(fr, sub_(tb.z, ta.z), ta.z), C3 = fma_(fr, sub_(tb.w, ta.w), ta.w);
+        if (above) {
+            C0 = tb.x; C1 = tb.y; C2 = tb.z; C3 = tb.w;
             atomicAdd(&sC[CNT_CLAMP + 0], 1u);
-        } else {
-            const int i = (int)xi;
-            const T fr = sub_(xi, (T)i);
-            const Row4 a = Te[i], b = Te[i + 1];
-            C0 = fma_(fr, sub_(b.x, a.x), a.x);
-            C1 = fma_(fr, sub_(b.y, a.y), a.y);
-            C2 = fma_(fr, sub_(b.z, a.z), a.z);
-            C3 = fma_(fr, sub_(b.w, a.w), a.w);
         }
         const T R = mul_((T)u01(r.y), K.kmax_e);
         const int j = (R < C0) ? 0 : (R < C1) ? 1 : (R < C2) ? 2 : (R < C3) ? 3 : 4;
@@ -290,7 +331,7 @@ __device__ __forceinline__ uint32_t collide(const Seg<T>& S, Cand<T>& q, int qc,
             // the scattered electron's direction: the same draw for every process, so it is
             // formed once, outside the per-process branches
             T nx, ny, nz;
-            iso_dir(u01(r.z), u01(r.w), nx, ny, nz);
+            direction(u01(r.z), u01(r.w), nx, ny, nz);
             if (j == 0) {  // elastic, target at rest: v' = beta v + (1-beta)|v| n
                 const T g = sqrt_(e2);
                 const T og = mul_(K.omb, g);
@@ -316,15 +357,15 @@ __device__ __forceinline__ uint32_t collide(const Seg<T>& S, Cand<T>& q, int qc,
                     vx = mul_(sp, nx);
                     vy = mul_(sp, ny);
                     vz = mul_(sp, nz);
-                    const U4 q1 = draw(seed, slot, step, 0, 1, S.did);
-                    const U4 w = draw(seed, slot, step, 0, 2, S.did);
-                    iso_dir(u01(q1.x), u01(q1.y), nx, ny, nz);
+                    const U4 q1 = rs.draw(slot, 1);
+                    const U4 w = rs.draw(slot, 2);
+                    direction(u01(q1.x), u01(q1.y), nx, ny, nz);
                     cvx = mul_(sp, nx);
                     cvy = mul_(sp, ny);
                     cvz = mul_(sp, nz);
                     float b0, b1, b2, b3;
-                    box_muller(u01(q1.z), u01(q1.w), b0, b1);
-                    box_muller(u01(w.x), u01(w.y), b2, b3);
+                    normals(u01(q1.z), u01(q1.w), b0, b1);
+                    normals(u01(w.x), u01(w.y), b2, b3);
                     ivx = mul_(K.sig_n, (T)b0);
                     ivy = mul_(K.sig_n, (T)b1);
                     ivz = mul_(K.sig_n, (T)b2);
@@ -342,7 +383,7 @@ __device__ __forceinline__ uint32_t collide(const Seg<T>& S, Cand<T>& q, int qc,
             int side = drift(N, K.dtdx, qc, qf, cvz, cn, fn, err);
             if (side < 0) {
                 store_rec<T>(S.sc, S.sp_, ridx, Part<T>{cn, fn, cvx, cvy, cvz});
-                dep_add(sH, cn, cic_F(fn));
+                dep_add(sH, cn, cic_F(fn), threadIdx.x & 31);
                 out |= 2u;
             } else {
                 atomicAdd(&sC[CNT_ABS + side], 1u);
@@ -351,18 +392,18 @@ __device__ __forceinline__ uint32_t collide(const Seg<T>& S, Cand<T>& q, int qc,
             side = drift(N, K.dtdx, qc, qf, ivz, cn, fn, err);
             if (side < 0) {
                 store_rec<T>(S.bc, S.bp, ridx, Part<T>{cn, fn, ivx, ivy, ivz});
-                hist_add(S.Dother, cn, cic_F(fn));
+                hist_add(Dother, cn, cic_F(fn));
                 out |= 4u;
             } else {
                 atomicAdd(&sC[CNT_ABS + 2 + side], 1u);
             }
         }
     } else {
-        const U4 r = draw(seed, slot, step, 1, 0, S.did);
-        const U4 q1 = draw(seed, slot, step, 1, 1, S.did);
+        const U4 r = rs.draw(slot, 0);
+        const U4 q1 = rs.draw(slot, 1);
         float a0, a1, a2, a3;
-        box_muller(u01(q1.x), u01(q1.y), a0, a1);
-        box_muller(u01(q1.z), u01(q1.w), a2, a3);
+        normals(u01(q1.x), u01(q1.y), a0, a1);
+        normals(u01(q1.z), u01(q1.w), a2, a3);
         const T vnx = mul_(K.sig_n, (T)a0), vny = mul_(K.sig_n, (T)a1), vnz = mul_(K.sig_n, (T)a2);
         const T gx = sub_(vx, vnx), gy = sub_(vy, vny), gz = sub_(vz, vnz);
         const T g2 = fma_(gx, gx, fma_(gy, gy, mul_(gz, gz)));
@@ -384,7 +425,7 @@ __device__ __forceinline__ uint32_t collide(const Seg<T>& S, Cand<T>& q, int qc,
         if (R < C0) {  // isotropic in the centre-of-mass frame, equal masses
             const T hg = mul_((T)0.5, sqrt_(g2));
             T nx, ny, nz;
-            iso_dir(u01(r.z), u01(r.w), nx, ny, nz);
+            direction(u01(r.z), u01(r.w), nx, ny, nz);
             vx = fma_(hg, nx, mul_(add_(vx, vnx), (T)0.5));
             vy = fma_(hg, ny, mul_(add_(vy, vny), (T)0.5));
             vz = fma_(hg, nz, mul_(add_(vz, vnz), (T)0.5));
@@ -404,18 +445,18 @@ __device__ __forceinline__ uint32_t collide(const Seg<T>& S, Cand<T>& q, int qc,
 
 // Secondary electron of an ion absorbed at electrode `side` (added option).
 template <typename T>
-__device__ __forceinline__ bool emit_see(const Seg<T>& S, uint32_t slot, long long step, unsigned long long seed,
+__device__ __forceinline__ bool emit_see(const Seg<T>& S, unsigned long long* Dother, uint32_t slot, const Stream& rs,
                                       int side, Part<T>& p, unsigned* sC) {
     const Consts<T>& K = S.k;
-    const U4 w = draw(seed, slot, step, 1, 3, S.did);
+    const U4 w = rs.draw(slot, 3);
     if (!((T)u01(w.x) < K.gamma)) return false;
     const T vn = mul_(K.sig_see_n, (T)__fsqrt_rn(-own_logf(u01(w.y))));
     float t0, t1;
-    box_muller(u01(w.z), u01(w.w), t0, t1);
+    normals(u01(w.z), u01(w.w), t0, t1);
     const int ce = side == 0 ? 0 : S.N - 1;
     const T fe = side == 0 ? (T)0 : one_minus_ulp<T>();
     p = Part<T>{ce, fe, mul_(K.sig_see, (T)t0), mul_(K.sig_see, (T)t1), side == 0 ? vn : -vn};
-    hist_add(S.Dother, ce, cic_F(fe));
+    hist_add(Dother, ce, cic_F(fe));
     atomicAdd(&sC[CNT_SEE], 1u);
     atomicAdd(&sC[CNT_SEE_SIDE + side], 1u);
     return true;
@@ -432,6 +473,12 @@ __device__ __forceinline__ void move_rec(int32_t* c, void* p, unsigned src, unsi
     c[dst] = cv;
     pp[dst] = rv;
 }
+
+// n mod m and n / m for step numbers (32-bit operations below 2^31, the slow 64-bit ones out of line).
+__device__ __noinline__ int mod_slow(long long n, int m) { return (int)(n % m); }
+__device__ __noinline__ long long div_slow(long long n, int m) { return n / m; }
+__device__ __forceinline__ int step_mod(long long n, int m) { return n >> 31 ? mod_slow(n, m) : (int)((unsigned)n % (unsigned)m); }
+__device__ __forceinline__ long long step_div(long long n, int m) { return n >> 31 ? div_slow(n, m) : (unsigned)n / (unsigned)m; }
 
 // Store totals after a sweep, for discharge d, by one warp of k_post: from the slice sums of parity
 // par, the new counts and the layout of the output buffer (the sweep's chunks become its regions,
@@ -450,13 +497,13 @@ __device__ __forceinline__ void store_totals(const Disc& D, int d, Ctl* ctl, int
     long long main0 = 0, main1 = 0, same0 = 0, see = 0, ions = 0;
     for (long long k = lane; k < max(slices[0], slices[1]); k += 32) {
         if (k < slices[0]) {
-            main0 += T0[3 * k + 0];
-            ions += T0[3 * k + 1];
-            same0 += T0[3 * k + 2];
+            main0 += __ldcg(T0 + 3 * k + 0);
+            ions += __ldcg(T0 + 3 * k + 1);
+            same0 += __ldcg(T0 + 3 * k + 2);
         }
         if (k < slices[1]) {
-            main1 += T1[3 * k + 0];
-            see += T1[3 * k + 1];
+            main1 += __ldcg(T1 + 3 * k + 0);
+            see += __ldcg(T1 + 3 * k + 1);
         }
     }
 #pragma unroll
@@ -491,8 +538,8 @@ __device__ __forceinline__ void store_totals(const Disc& D, int d, Ctl* ctl, int
             if (full_step) {  // per-period mean counts (steady-state criterion)
                 const long long n_step = ctl->step;  // this step is n; the counts belong to n+1
                 ctl->period_acc[d][sp] += (double)n_new;
-                if (D.steps_per_period > 0 && (n_step + 1) % D.steps_per_period == 0) {
-                    const long long per = (n_step + 1) / D.steps_per_period - 1;
+                if (D.steps_per_period > 0 && step_mod(n_step + 1, D.steps_per_period) == 0) {
+                    const long long per = step_div(n_step + 1, D.steps_per_period) - 1;
                     D.period_mean[(per % PERIOD_HIST) * 2 + sp] = ctl->period_acc[d][sp] / D.steps_per_period;
                     ctl->period_acc[d][sp] = 0.0;
                 }
@@ -535,351 +582,385 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* mb, unsigned parit
     return false;
 }
 
-// Dynamic shared memory of the sweep: the node field (T, N+1), the deposit histogram (u32 n, lo, hi
-// per cell) and the energy moment (u32 lo, hi per node); per warp two staging buffers of one chunk (records, then cells) and its candidate
-// queue; per store the layout snapshot and the tile prefix.
-template <typename T>
-__host__ __device__ constexpr size_t sweep_hist_offset(int max_N) {  // after the node field
-    return (((size_t)(max_N + 1) * sizeof(T) + 15) / 16) * 16;
+// Dynamic shared memory of the sweep: per cell the field and its difference to the next node (E_c,
+// E_{c+1} - E_c), the histograms (`sets` 2: both species at once, 5 + 3 arrays; 1: one species at a
+// time, 5 arrays) and their windows, per warp two staging buffers of one chunk (records, then cells) and its candidate
+// queue, per store its layout, per species the chunk prefix over the discharges.
+struct StoreSnap {
+    int K, chunks, M, D0, n;
+};
+template <typename T, int PPT>
+__host__ __device__ constexpr unsigned sweep_stage_bytes() {  // one buffer of one warp
+    return 32u * PPT * (sizeof(typename Rec<T>::type) + 4);
 }
+__host__ __device__ constexpr int sweep_hist_words(int sets) { return sets == 2 ? 8 : 5; }
 template <typename T>
-__host__ __device__ constexpr size_t sweep_stage_offset(int max_N) {
-    return ((sweep_hist_offset<T>(max_N) + 4 * (3 * (size_t)max_N + 2 * ((size_t)max_N + 1)) + 127) / 128) * 128;
+__host__ __device__ constexpr unsigned sweep_hist_offset(int max_N) { return (2u * sizeof(T) * max_N + 15) / 16 * 16; }
+template <typename T>
+__host__ __device__ constexpr unsigned sweep_stage_offset(int max_N, int sets) {
+    return (sweep_hist_offset<T>(max_N) + 4u * sweep_hist_words(sets) * (max_N + WWORDS) + 127) / 128 * 128;
 }
 template <typename T, int PPT>
-__host__ __device__ constexpr size_t sweep_stage_bytes() {  // one buffer of one warp
-    return (size_t)32 * PPT * (sizeof(typename Rec<T>::type) + 4);
-}
-template <typename T, int BLOCK, int PPT>
-__host__ __device__ constexpr size_t sweep_queue_offset(int max_N) {
-    return sweep_stage_offset<T>(max_N) + 2 * (BLOCK / 32) * sweep_stage_bytes<T, PPT>();
-}
-template <typename T, int BLOCK, int PPT>
-__host__ __device__ constexpr size_t sweep_store_offset(int max_N) {
-    return ((sweep_queue_offset<T, BLOCK, PPT>(max_N) + (size_t)BLOCK * PPT + 15) / 16) * 16;
-}
-struct StoreSnap {  // layout of one input store, for the prefetches of any tile
-    int K, chunks;
-    long long M, D0, n;
-};
-template <typename T, int BLOCK, int PPT>
-__host__ __device__ constexpr size_t sweep_smem(int max_N, int n_disc) {
-    return sweep_store_offset<T, BLOCK, PPT>(max_N) + sizeof(StoreSnap) * 2 * (size_t)n_disc +
-           sizeof(long long) * (2 * (size_t)n_disc + 1);
+__host__ __device__ constexpr unsigned sweep_smem(int max_N, int sets, int warps, int n_disc) {
+    return sweep_stage_offset<T>(max_N, sets) + (unsigned)warps * (2 * sweep_stage_bytes<T, PPT>() + 32 * PPT) +
+           (unsigned)sizeof(StoreSnap) * 2 * n_disc + 4u * 2 * (n_disc + 1);
 }
 
-// Resident threads per SM the sweep is compiled for (the register budget is 65536 / that): the
-// FP32 chunk state fits 64 registers at PPT <= 2 and 80 at PPT = 4; 512-thread CTAs at PPT = 4 are
-// held to 64 registers so that two of them fit an SM.
-template <typename T, int BLOCK, int PPT>
-__host__ __device__ constexpr int sweep_threads_per_sm() {
-    return sizeof(T) == 4 ? (PPT <= 2 ? 1024 : PPT == 4 ? (BLOCK >= 512 ? 1024 : 768) : 512) : 256;
-}
-template <typename T, int BLOCK, int PPT>
-__host__ __device__ constexpr int sweep_min_blocks() {
-    return sweep_threads_per_sm<T, BLOCK, PPT>() / BLOCK > 0 ? sweep_threads_per_sm<T, BLOCK, PPT>() / BLOCK : 1;
-}
+// Threads of a sweep CTA at most (one CTA per SM): the FP32 chunk code takes 80 registers (24 warps), the
+// FP64 code 128 (16 warps).
+template <typename T>
+__host__ __device__ constexpr int sweep_max_threads() { return sizeof(T) == 4 ? 768 : 512; }
 
 // ---------------------------------------------------------------------------
-// The sweep. Persistent CTAs take the tiles of NW chunks of all stores (discharge, species) in a
-// static grid-stride order; warp w of a tile owns the tile's chunk w (at most CHUNK = 32 PPT
-// slots, a region or a run of the dense part of the input layout) and works on it alone, with no
-// barrier: the chunk's records and cells arrive in the warp's staging buffer by a bulk copy issued
-// while the warp was processing its previous chunk; the warp pushes its particles (gather, kick,
-// energy moment, candidate test), runs one collision pass over the chunk's candidates, then kicks,
-// drifts, deposits and writes the survivors in slot order to the chunk's own output region
-// [CHUNK cs, ...), cs the chunk index. Newborns go in parent-slot order to the chunk's regions of
-// the newborn buffers (same species: ionization electrons; other species: ionization ions, or SEE
-// electrons of the ion sweep), and the chunk records the three counts. The CTA synchronises only
-// where its tiles move to another store (histogram flush).
-template <typename T, int BLOCK, int PPT>
-__global__ void __launch_bounds__(BLOCK, sweep_min_blocks<T, BLOCK, PPT>())
+// The sweep. One persistent CTA per SM. The chunks of all electron stores and those of all ion stores
+// are split evenly over the CTAs (CTA b takes the contiguous chunks [total b / G, total (b+1) / G) of
+// each list), and each CTA's part of a store over its warps, again contiguous. So a CTA meets few
+// stores, its deposits few cells, and consecutive chunks of a warp share a candidate call.
+// A chunk's records and cells arrive in the warp's staging buffer by a bulk copy issued while the warp
+// worked on its previous chunk; the warp draws the chunk's candidate words and queues the candidates in
+// slot order; collides them (32 at a time, the final velocity written back into the staged record, the
+// staged cell marked COLLIDED); then takes all particles in one pass: gather, half kicks, energy moment,
+// drift, walls, deposit, survivors in slot order to the chunk's own output region [CHUNK cs, ...), cs the
+// chunk index. Newborns go in parent-slot order to the chunk's regions of the newborn buffers (same
+// species: ionization electrons; other species: ionization ions, or SEE electrons of the ion sweep), and
+// the chunk records the three counts. The CTA synchronises only between discharges (with one histogram
+// set, between stores) and for a flush of its histograms.
+//
+// What bounds it: instruction issue, then the shared-memory atomics; for a store of a few chunks per SM
+// the latency of one chunk (cold instructions, table look-ups, 40 % of it the collisions). Measured, with
+// the FP32 chunk of 128 slots at 80 registers and 24 warps (32 warps at 64 registers spill: 40.5 against
+// 35.7 us a step at 1e6 + 1e6 and 392 against 320 at 1.2e7 + 1.2e7): 31 us a launch at 1e6 + 1e6
+// particles, 512 cells (before: one CTA of 8 warps per 1024 slots, three passes over a chunk and a gather
+// in each, 40 us), 262 at 1.2e7 + 1.2e7, 2048 cells (372), 58 for 64 discharges of 2e4 + 2e4 in one launch
+// (109), FP64 at 1e6 + 1e6 90 (150).
+template <typename T, int PPT>
+__global__ void __launch_bounds__(sweep_max_threads<T>(), 1)
     k_sweep(const Disc* __restrict__ discs, int n_disc, Ctl* __restrict__ ctl, int in_buf, unsigned long long seed,
-            int max_N) {
+            int max_N, int sets) {
     using R = typename Rec<T>::type;
-    constexpr int NW = BLOCK / 32;
+    using T2 = typename T4<T>::two;
     constexpr int CHUNK = 32 * PPT;
     constexpr unsigned REC_BYTES = CHUNK * sizeof(R), CELL_BYTES = CHUNK * 4;
+    constexpr int COLLIDED = 1 << 30;  // mark in a staged cell: the record holds the particle's final velocity
+    constexpr int MAXW = sweep_max_threads<T>() / 32;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    T* s_E = reinterpret_cast<T*>(smem_raw);
-    unsigned* s_h32 = reinterpret_cast<unsigned*>(smem_raw + sweep_hist_offset<T>(max_N));
-    const DepHist s_dep{s_h32, s_h32 + max_N, s_h32 + 2 * max_N};
-    unsigned* s_qlo = s_h32 + 3 * max_N;
-    unsigned* s_qhi = s_qlo + (max_N + 1);
-    const int h32_words = 3 * max_N + 2 * (max_N + 1);
-    StoreSnap* s_store = reinterpret_cast<StoreSnap*>(smem_raw + sweep_store_offset<T, BLOCK, PPT>(max_N));
-    long long* s_segstart = reinterpret_cast<long long*>(s_store + 2 * n_disc);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthr = blockDim.x, NW = nthr >> 5;
+    T2* s_E = reinterpret_cast<T2*>(smem_raw);
+    unsigned* s_win = reinterpret_cast<unsigned*>(smem_raw + sweep_hist_offset<T>(max_N));  // 16-byte aligned
+    unsigned* s_h = s_win + sweep_hist_words(sets) * WWORDS;
+    unsigned char* s_stage = smem_raw + sweep_stage_offset<T>(max_N, sets);
+    unsigned char* stage = s_stage + (unsigned)warp * 2 * sweep_stage_bytes<T, PPT>();
+    unsigned char* s_queue = s_stage + (unsigned)NW * 2 * sweep_stage_bytes<T, PPT>();
+    uint8_t* Q = s_queue + warp * CHUNK;  // the chunk indices of the candidates, in slot order (CHUNK <= 256)
+    StoreSnap* s_store = reinterpret_cast<StoreSnap*>(s_queue + NW * CHUNK);
+    int* s_pre = reinterpret_cast<int*>(s_store + 2 * n_disc);  // [species][n_disc + 1]
 
-    __shared__ Seg<T> S;
+    __shared__ Seg<T> s_seg[2];
     __shared__ long long s_step;
-    __shared__ int s_par;
+    __shared__ int s_par, s_dpar;  // parities of the slice sums and of the deposits
     __shared__ unsigned s_cnt[NCNT];
     __shared__ int s_err;
-    __shared__ unsigned long long s_mbar[NW][2];
-    // per warp: the chunk prefetched for its next tile (chunk index, first and end slot, valid), the
-    // store of the last prefetch, and the barrier phases (kept here, not in registers)
-    __shared__ int s_pf[NW][6];
+    __shared__ unsigned long long s_mbar[MAXW][2];
+    __shared__ int2 s_range[2 * MAXD];
+    __shared__ unsigned s_mask[4];
+    __shared__ int s_w0[2];  // first cell of each species' window
 
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    unsigned char* stage = smem_raw + sweep_stage_offset<T>(max_N) + (size_t)warp * 2 * sweep_stage_bytes<T, PPT>();
-    // per warp: the chunk indices of its candidates, in slot order (CHUNK <= 256)
-    uint8_t* Q = reinterpret_cast<uint8_t*>(smem_raw + sweep_queue_offset<T, BLOCK, PPT>(max_N)) + warp * CHUNK;
     if (lane == 0) {
         mbar_init(&s_mbar[warp][0]);
         mbar_init(&s_mbar[warp][1]);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    // the two stores' constants of discharge d
+    auto load_seg = [&](int d) {
+        const unsigned* src = reinterpret_cast<const unsigned*>(segs_of<T>(discs[d]));
+        unsigned* dst = reinterpret_cast<unsigned*>(s_seg);
+        for (int j = tid; j < (int)(sizeof(s_seg) / 4); j += nthr) dst[j] = __ldg(src + j);
+    };
+    if (tid == 0) s_err = 0;
+    if (tid < NCNT) s_cnt[tid] = 0;
+    load_seg(0);  // of a context with one discharge: nothing more to fetch after the wait
+    for (int j = tid; j < sweep_hist_words(sets) * (max_N + WWORDS); j += nthr) s_win[j] = 0;
+    __syncthreads();
     grid_dep_sync();
-    if (tid == 0) {
-        long long acc = 0;
-        int err0 = 0;
-        for (int s = 0; s < 2 * n_disc; ++s) {
-            const int d = s >> 1, sp = s & 1;
-            const Lay L = ctl->lay[d][sp][in_buf];
-            const long long n = ctl->count[d][sp];
-            long long ch = chunks_of(L, n, CHUNK);
-            if (ch > discs[d].ralloc[sp]) {  // more chunks than output regions: reported, the rest dropped
-                ch = discs[d].ralloc[sp];
-                err0 |= ERR_CAPACITY;
-            }
-            s_store[s] = StoreSnap{L.K, (int)ch, L.M, L.D0, n};
-            s_segstart[s] = acc;
-            acc += (ch + NW - 1) / NW;
-            if (blockIdx.x == 0) ctl->chunks_in[d][sp] = (int)ch;  // read by the post-sweep grid
+    auto load_field = [&]() {
+        const T* E = reinterpret_cast<const T*>(s_seg[0].E);
+        const int N = s_seg[0].N;
+        for (int j = tid; j < N; j += nthr) {
+            const T e0 = __ldcg(E + j), e1 = __ldcg(E + j + 1);
+            T2 v;
+            v.x = e0;
+            v.y = sub_(e1, e0);
+            s_E[j] = v;
         }
-        s_segstart[2 * n_disc] = acc;
+    };
+    // every store's layout; 31 bits hold slots, chunks and record offsets (the host caps the buffers)
+    const int n_store = 2 * n_disc;
+    for (int s = tid; s < n_store; s += nthr) {
+        const int d = s >> 1, sp = s & 1;
+        const Lay L = ctl->lay[d][sp][in_buf];
+        const long long n = ctl->count[d][sp];
+        long long ch = chunks_of(L, n, CHUNK);
+        if (ch > discs[d].ralloc[sp]) {  // more chunks than output regions: reported, the rest dropped
+            ch = discs[d].ralloc[sp];
+            if (blockIdx.x == 0) atomicOr(&s_err, ERR_CAPACITY);
+        }
+        s_store[s] = StoreSnap{L.K, (int)ch, (int)L.M, (int)L.D0, (int)n};
+        if (blockIdx.x == 0) ctl->chunks_in[d][sp] = (int)ch;  // read by the post-sweep grid
+        s_pre[sp * (n_disc + 1) + d + 1] = (int)ch;
+        if (d == 0) s_pre[sp * (n_disc + 1)] = 0;
+    }
+    if (tid == 0) {
         s_step = ctl->step;
         s_par = ctl->slice_par;
-        s_err = blockIdx.x == 0 ? err0 : 0;
+        s_dpar = ctl->dep_par;
+    }
+    if (n_disc == 1) load_field();
+    if (n_disc > 1) {  // inclusive prefix over at most 64 discharges: warp sp takes its species, two per lane
+        __syncthreads();
+        if (warp < 2) {
+            int* p = s_pre + warp * (n_disc + 1) + 1;
+            const int v0 = 2 * lane < n_disc ? p[2 * lane] : 0, v1 = 2 * lane + 1 < n_disc ? p[2 * lane + 1] : 0;
+            int x = v0 + v1;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(FULL, x, o);
+                if (lane >= o) x += y;
+            }
+            if (2 * lane < n_disc) p[2 * lane] = x - v1;
+            if (2 * lane + 1 < n_disc) p[2 * lane + 1] = x;
+        }
+        __syncthreads();
+    }
+    // this CTA's chunks [lo, hi) of every store (electrons and ions of a discharge in turn) and the bits
+    // of the stores it has any of
+    auto take = [&](int t) {  // warp-uniform trip counts: every lane calls
+        int lo = 0, hi = 0;
+        if (t < n_store) {
+            const int* p = s_pre + (t & 1) * (n_disc + 1);
+            const unsigned tot = (unsigned)p[n_disc], G = gridDim.x, b = blockIdx.x;
+            const unsigned w = tot / G, x = tot - w * G;  // the first x CTAs take w + 1 chunks
+            const int r0 = (int)(b * w + min(b, x)), r1 = r0 + (int)(w + (b < x ? 1 : 0));
+            const int p0 = p[t >> 1], p1 = p[(t >> 1) + 1];
+            lo = min(max(r0, p0), p1) - p0;
+            hi = min(max(r1, p0), p1) - p0;
+            s_range[t] = make_int2(lo, hi);
+        }
+        const unsigned m = __ballot_sync(FULL, hi > lo);
+        if (lane == 0) s_mask[t >> 5] = m;
+    };
+    if (n_disc == 1) {
+        if (warp == 0) {
+            __syncwarp();
+            take(lane);
+        }
+    } else {
+        for (int t = tid; t < 2 * MAXD; t += nthr) take(t);
     }
     __syncthreads();
-    const int total_tiles = (int)s_segstart[2 * n_disc];  // tiles and chunks fit in 31 bits (record offsets do)
     const long long step = s_step;
-    int cur_seg = -1, cur_d = -1;
-    int err = 0;
-
-    // Adds the CTA's histograms and counters of the current store to the global ones and clears them.
-    auto flush = [&]() {
-        __syncthreads();
-        const int N = S.N;
-        for (int j = tid; j <= N; j += BLOCK) {
-            unsigned long long h = 0;
-            if (j < N)
-                h = ((unsigned long long)s_dep.n[j] << 32) -
-                    ((unsigned long long)s_dep.lo[j] + ((unsigned long long)s_dep.hi[j] << 16));
-            if (j > 0) h += (unsigned long long)s_dep.lo[j - 1] + ((unsigned long long)s_dep.hi[j - 1] << 16);
-            if (h) atomicAdd(&S.Dg[j], h);
-            if (S.sp == 0) {
-                const unsigned long long q = (unsigned long long)s_qlo[j] + ((unsigned long long)s_qhi[j] << 13);
-                if (q) atomicAdd(&S.Qg[j], q);
-            }
-        }
-        if (tid < NCNT && s_cnt[tid]) atomicAdd(&S.cnt[tid], (unsigned long long)s_cnt[tid]);
-        __syncthreads();
-        for (int j = tid; j < h32_words; j += BLOCK) s_h32[j] = 0;
-        if (tid < NCNT) s_cnt[tid] = 0;
-        __syncthreads();
+    // the next store after s (-1: the first) that this CTA has chunks of, n_store if none
+    auto next_store = [&](int s) {
+        ++s;
+        unsigned m = s < n_store ? s_mask[s >> 5] >> (s & 31) : 0u;
+        if (m) return s + __ffs(m) - 1;
+        for (int w = (s >> 5) + 1; 32 * w < n_store; ++w)
+            if (s_mask[w]) return 32 * w + __ffs(s_mask[w]) - 1;
+        return n_store;
+    };
+    // this warp's part of them; the ions in the opposite warp order, so that a warp with one chunk more
+    // of one species tends to have one less of the other
+    auto warp_range = [&](int s, int& lo, int& hi) {
+        const int2 r = s_range[s];
+        const unsigned w = (s & 1) ? NW - 1 - warp : warp, m = r.y - r.x, q = m / NW, x = m % NW;
+        lo = r.x + (int)(w * q + min(w, x));
+        hi = lo + (int)(q + (w < x ? 1 : 0));
     };
 
-    // Prefetch of this warp's chunk of tile gn into staging buffer b: the store of the tile, the
-    // chunk's record offset (known without any table) and its first and end slot (regions: from
-    // the start table, loaded now and used when the chunk is processed).
-    int* pf = s_pf[warp];  // [0] chunk, [1] first slot, [2] end slot, [3] valid, [4] store, [5] phases
-    auto prefetch = [&](int b, int gn) {
-        if (lane == 0) pf[3] = 0;
-        if (gn >= total_tiles) return;
-        int sg = pf[4];
-        while (sg + 1 < 2 * n_disc && s_segstart[sg + 1] <= gn) ++sg;
-        const StoreSnap ss = s_store[sg];
-        const int cs = (gn - (int)s_segstart[sg]) * NW + warp;
-        if (cs >= ss.chunks) return;
-        const int d = sg >> 1, sp = sg & 1;
-        long long src;
-        int pst0, pst1;
-        if (cs < ss.K) {
-            src = (long long)cs * CHUNK;
-            const int* st = discs[d].start[sp];
-            pst0 = __ldg(st + cs);
-            pst1 = __ldg(st + cs + 1);
+    // the chunk whose copy is in flight (or landed) in buffer pf_b: its store (n_store: none), index,
+    // the warp's last chunk of that store, first and end slot
+    int pf_s = -1, pf_k = 0, pf_end = 0, pf_base = 0, pf_stop = 0, pf_b = 1;
+    unsigned phases = 0;  // bit b: phase of buffer b's barrier the next wait expects
+    auto prefetch_next = [&]() {
+        ++pf_k;
+        while (pf_k >= pf_end) {
+            pf_s = next_store(pf_s);
+            if (pf_s >= n_store) return;
+            warp_range(pf_s, pf_k, pf_end);
+        }
+        pf_b ^= 1;
+        const StoreSnap ss = s_store[pf_s];
+        const Seg<T>& G = n_disc == 1 ? s_seg[pf_s] : segs_of<T>(discs[pf_s >> 1])[pf_s & 1];
+        unsigned src;
+        if (pf_k < ss.K) {
+            src = (unsigned)pf_k * CHUNK;
+            const int* st = G.start + pf_k;
+            pf_base = __ldcg(st);
+            pf_stop = __ldcg(st + 1);
         } else {
-            const long long j = (long long)(cs - ss.K);
-            src = ss.D0 + j * CHUNK;
-            pst0 = (int)(ss.M + j * CHUNK);
-            pst1 = (int)min(ss.n, ss.M + (j + 1) * CHUNK);
+            const int j = (pf_k - ss.K) * CHUNK;
+            src = (unsigned)(ss.D0 + j);
+            pf_base = ss.M + j;
+            pf_stop = min(ss.n, pf_base + CHUNK);
         }
         if (lane == 0) {
-            pf[0] = (int)cs;
-            pf[1] = pst0;
-            pf[2] = pst1;
-            pf[3] = 1;
-            pf[4] = sg;
-            unsigned char* buf = stage + (size_t)b * sweep_stage_bytes<T, PPT>();
+            unsigned char* buf = stage + (unsigned)pf_b * sweep_stage_bytes<T, PPT>();
+            unsigned long long* mb = &s_mbar[warp][pf_b];
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // earlier reads and writes of the buffer
-            mbar_expect(&s_mbar[warp][b], REC_BYTES + CELL_BYTES);
-            bulk_g2s(buf, reinterpret_cast<const R*>(discs[d].p[in_buf][sp]) + src, REC_BYTES, &s_mbar[warp][b]);
-            bulk_g2s(buf + REC_BYTES, discs[d].c[in_buf][sp] + src, CELL_BYTES, &s_mbar[warp][b]);
+            mbar_expect(mb, REC_BYTES + CELL_BYTES);
+            bulk_g2s(buf, reinterpret_cast<const R*>(G.p[in_buf]) + src, REC_BYTES, mb);
+            bulk_g2s(buf + REC_BYTES, G.c[in_buf] + src, CELL_BYTES, mb);
         }
     };
+    prefetch_next();
 
     const unsigned lt = (1u << lane) - 1u;
-    if (lane == 0) {
-        pf[4] = 0;
-        pf[5] = 0;  // bit b: phase of buffer b's barrier the next wait expects
-    }
-    __syncwarp();
-    prefetch(0, blockIdx.x);  // the chunk of the CTA's first tile, into buffer 0
-    __syncwarp();
+    int err = 0;
+    unsigned carry = 0, carry_q = 0xFFFFFFFFu;  // candidate bits of the last call of the warp's previous chunk
 
-    // One warp's chunk of the store of species SP: push, collide, write (see above). Phases B and C
-    // read each particle again from the staging buffer and repeat the gather and the first half kick
-    // (the same operations, so the same values) instead of keeping them in registers or in the
-    // queue; a collision writes the velocity after it back into the staged record, and phase C then
-    // takes that velocity as v_n.
-    auto chunk = [&](unsigned cs, int base, int cnt, R* srec, const int32_t* scell, auto spc) {
-        constexpr int SP = decltype(spc)::value;
+    // One warp's chunk of the store of species SP (see above).
+    auto chunk = [&](unsigned cs, int base, int cnt, R* srec, int32_t* scell, auto spc) { constexpr int SP = decltype(spc)::value;
+        const Seg<T>& S = s_seg[SP];
+        const int h0 = SP == 1 && sets == 2 ? 5 : 0;
+        const Hist h{s_h + h0 * max_N, s_win + h0 * WWORDS, max_N, s_w0[SP]};
         const unsigned obase = cs * CHUNK;
         unsigned offA = obase, offB = obase, offS = obase;  // output cursors of the chunk's regions
         const int N = S.N;
         const T Ksp = S.k.K[SP];
-        // particle i of the chunk: cell (-1 if none or out of range), offset, velocity, gathered field
-        auto particle = [&](int i, int& c, T& f, T& vx, T& vy, T& vz, T& ef) {
-            c = -1;
-            f = vx = vy = vz = ef = (T)0;
-            if (i < cnt) {
-                c = scell[i];
-                const R r = srec[i];
-                f = r.x;
-                vx = r.y;
-                vy = r.z;
-                vz = r.w;
-                if (!((unsigned)c < (unsigned)N)) c = -1;
-                else {
-                    const T E0 = s_E[c], E1 = s_E[c + 1];
-                    ef = fma_(f, sub_(E1, E0), E0);
+        const Stream rs{seed, (uint32_t)step, ((uint32_t)((unsigned long long)step >> 32) & 0xFFFFu) << 16 | (uint32_t)SP << 8,
+                        S.did};
+        if (cnt > 0) {
+            // ---- candidates. Slots 4q..4q+3 take the four words of one Philox call (call 4, counter
+            // word 0 = q) and are candidates where a word is below the threshold. The chunk needs the
+            // calls q0 .. (base + cnt - 1) / 4; the first is the previous chunk's last one when that
+            // chunk's slots run into this one's, so its bits are carried over and 32 calls cover 128
+            // slots at any alignment.
+            constexpr int NG = (CHUNK / 4 + 1 + 31) / 32;
+            const unsigned q0 = (unsigned)base >> 2;
+            const int al = base & 3;
+            const int ncalls = (int)(((unsigned)base + cnt - 1) >> 2) - (int)q0 + 1;
+            const int sh = carry_q == q0 ? 1 : 0;
+            int qn = 0;
+            if (sh) {  // words al.. of the carried call: chunk indices 0..3 - al
+                const unsigned cm = (carry >> al) & ((1u << min(cnt, 4 - al)) - 1u);
+                if (cm) {
+                    if (lane < 4 && ((cm >> lane) & 1u)) Q[__popc(cm & lt)] = (uint8_t)lane;
+                    qn = __popc(cm);
                 }
             }
-        };
-        if (cnt > 0) {
-            // candidate words: slots 4q..4q+3 take the four words of one Philox call (call 4,
-            // counter word 0 = q); lane l computes the calls q0 + l + 32 m, q0 = base / 4, compares
-            // their words with the threshold and keeps the results as bits 4 m + w (word w); the
-            // particle of slot s takes bit s % 4 of call s / 4 by one shuffle
-            constexpr int NG = (CHUNK / 4 + 1 + 31) / 32;
-            const uint32_t did = S.did, thr = S.thr;
-            const unsigned q0 = (unsigned)base >> 2;
-            // calls needed: q0 .. (base + cnt - 1) / 4; the last group of calls is drawn only if the
-            // chunk reaches it (an unaligned first slot needs one call beyond CHUNK / 4)
-            const int ncalls = (int)(((unsigned)base + cnt - 1) >> 2) - (int)q0 + 1;
-            unsigned cbits = 0;
+            const int li = ncalls - 1 - sh;  // the last call is drawn by lane li % 32 of group li / 32
+            unsigned next = carry;
 #pragma unroll
             for (int m = 0; m < NG; ++m)
-                if (32 * m < ncalls) {
-                    const U4 w = draw(seed, q0 + lane + 32 * m, step, SP, 4, did);
-                    cbits |= ((w.x < thr ? 1u : 0u) | (w.y < thr ? 2u : 0u) | (w.z < thr ? 4u : 0u) |
-                              (w.w < thr ? 8u : 0u))
-                             << (4 * m);
-                }
-            // ---- phase A: gather, first half kick, energy moment, candidate test
-            unsigned candm = 0;  // bit k: this lane's particle of row k is a candidate
-            int qn = 0;
+                if (32 * m <= li) {
+                    const U4 w = rs.draw(q0 + sh + lane + 32 * m, 4);
+                    const uint32_t thr = S.thr;
+                    unsigned nib = (w.x < thr ? 1u : 0u) | (w.y < thr ? 2u : 0u) | (w.z < thr ? 4u : 0u) |
+                                   (w.w < thr ? 8u : 0u);
+                    if ((li >> 5) == m) next = __shfl_sync(FULL, nib, li & 31);
+                    // word k is chunk index i0 + k; only those in [0, cnt) count
+                    const int i0 = 4 * (lane + sh + 32 * m) - al;
+                    if (i0 < 0) nib &= 0xFu << -i0;
+                    const int left = cnt - i0;
+                    if (left < 4) nib = left > 0 ? nib & ((1u << left) - 1u) : 0u;
+                    if (__any_sync(FULL, nib != 0)) {
+                        const unsigned b0 = __ballot_sync(FULL, nib & 1u), b1 = __ballot_sync(FULL, nib & 2u),
+                                       b2 = __ballot_sync(FULL, nib & 4u), b3 = __ballot_sync(FULL, nib & 8u);
+                        int pos = qn + __popc(b0 & lt) + __popc(b1 & lt) + __popc(b2 & lt) + __popc(b3 & lt);
 #pragma unroll
-            for (int k = 0; k < PPT; ++k) {
-                const int i = 32 * k + lane;
-                int c;
-                T f, vx, vy, vz, ef;
-                particle(i, c, f, vx, vy, vz, ef);
-                if (i < cnt && c < 0) err |= ERR_NONFINITE;  // corrupt cell index: dropped and reported
-                const bool valid = c >= 0;
-                unsigned qa = 0, qb = 0;
-                if (valid) {
-                    vz = fma_(Ksp, ef, vz);  // v_n
-                    if (SP == 0) {  // energy moment at (x_n, v_n), 2^-12 eV, clamped at 2^26
-                        const T e2 = fma_(vx, vx, fma_(vy, vy, mul_(vz, vz)));
-                        T eq = mul_(e2, S.k.kappa_E);
-                        if (!(eq <= (T)0x1p26)) eq = (T)0x1p26;
-                        const unsigned long long Et = rint_u32(eq);
-                        const unsigned long long Eh = rint_u32(mul_(eq, f));
-                        qa = (unsigned)(Et - Eh);
-                        qb = (unsigned)Eh;
+                        for (int k = 0; k < 4; ++k)
+                            if ((nib >> k) & 1u) Q[pos++] = (uint8_t)(i0 + k);
+                        qn += __popc(b0) + __popc(b1) + __popc(b2) + __popc(b3);
                     }
                 }
-                if (SP == 0) warp_energy(s_qlo, s_qhi, c, qa, qb, lane);
-                const unsigned slot = (unsigned)base + i;
-                const unsigned r = (slot >> 2) - q0;
-                const unsigned cb = __shfl_sync(FULL, cbits, r & 31);
-                const bool cand = valid && ((cb >> (4 * (r >> 5) + (slot & 3))) & 1u);
-                const unsigned cm = __ballot_sync(FULL, cand);
-                if (lane == 0 && cm) atomicAdd(&s_cnt[CNT_CAND + SP], (unsigned)__popc(cm));
-                if (cand) {
-                    candm |= 1u << k;
-                    Q[qn + __popc(cm & lt)] = (uint8_t)i;
-                }
-                qn += __popc(cm);
-            }
-            // ---- phase B: the chunk's candidates, 32 at a time; newborns in queue (= slot) order
-            __syncwarp();
+            carry = next;
+            carry_q = q0 + ncalls - 1;
+            // ---- the candidates' collisions, 32 at a time; newborns in queue (= slot) order
+            if (qn) __syncwarp();
             for (int r0 = 0; r0 < qn; r0 += 32) {
                 const int q = r0 + lane;
                 uint32_t o = 0;
-                if (q < qn) {
-                    const int i = Q[q];
-                    int c;
-                    T f, vx, vy, vz, ef;
-                    particle(i, c, f, vx, vy, vz, ef);  // a candidate has a valid cell
-                    T vzc = fma_(Ksp, ef, vz);                 // v_n
-                    if (S.leapfrog) vzc = fma_(Ksp, ef, vzc);  // leapfrog: the collision acts on v_{n+1/2}
-                    Cand<T> e{ef, vx, vy, vzc};
-                    o = collide<T>(S, e, c, f, (uint32_t)base + i, obase + q, step, seed, s_dep, s_cnt, err);
-                    R& rec = srec[i];
-                    rec.y = e.vx;
-                    rec.z = e.vy;
-                    rec.w = e.vz;
+                const int i = Q[min(q, qn - 1)];
+                const int c0 = scell[i];
+                const bool cand = q < qn && (unsigned)c0 < (unsigned)N;  // a corrupt cell is dropped and reported below
+                const int c = cand ? c0 : 0;
+                R rec = srec[i];
+                const T2 e = s_E[c];
+                const T ef = fma_(rec.x, e.y, e.x);
+                const T vzn = fma_(Ksp, ef, rec.w);  // v_n
+                if (SP == 0)
+                    energy_add<T>(h, S.Qg, cand, c, rec.x, fma_(rec.y, rec.y, fma_(rec.z, rec.z, mul_(vzn, vzn))),
+                                  S.k.kappa_E, lane);
+                if (cand) {
+                    Cand<T> v{ef, rec.y, rec.z, S.leapfrog ? fma_(Ksp, ef, vzn) : vzn};  // leapfrog: at v_{n+1/2}
+                    o = collide<T>(S, SP, S.Dother + s_dpar * (N + 1), v, c, rec.x, (uint32_t)base + i, obase + q, rs, h, s_cnt, err);
+                    rec.y = v.vx;
+                    rec.z = v.vy;
+                    rec.w = S.leapfrog ? v.vz : fma_(Ksp, ef, v.vz);  // the second half kick
+                    srec[i] = rec;
+                    scell[i] = c | COLLIDED;
                 }
                 __syncwarp();
+                const unsigned mc = __ballot_sync(FULL, cand);
+                if (lane == 0 && mc) atomicAdd(&s_cnt[CNT_CAND + SP], (unsigned)__popc(mc));
                 if (SP == 0) {  // the round's newborns, from the candidates' ranks to parent-slot order (dst <= src)
                     const unsigned m1 = __ballot_sync(FULL, (o & 2u) != 0), m2 = __ballot_sync(FULL, (o & 4u) != 0);
-                    if (o & 2u) move_rec<T>(S.sc, S.sp_, obase + q, offS + __popc(m1 & lt));
-                    if (o & 4u) move_rec<T>(S.bc, S.bp, obase + q, offB + __popc(m2 & lt));
-                    offS += __popc(m1);
-                    offB += __popc(m2);
-                    __syncwarp();
-                }
-            }
-            // ---- phase C: second half kick, drift, walls, deposit, survivors in slot order
-            const T dtdx = S.k.dtdx;
-            int32_t* __restrict__ cout = S.cout;
-            void* pout = S.pout;
-#pragma unroll
-            for (int k = 0; k < PPT; ++k) {
-                const int i = 32 * k + lane;
-                bool alive = false, see = false;
-                Part<T> P0{}, Pse{};
-                int c;
-                T f, vx, vy, vz, ef;
-                particle(i, c, f, vx, vy, vz, ef);
-                if (c >= 0) {
-                    // v_n as in phase A; a candidate's staged record already holds its velocity after
-                    // the collision (at v_n, or at v_{n+1/2} in the leapfrog scheme, then final)
-                    const bool coll = (candm >> k) & 1u;
-                    if (!coll) vz = fma_(Ksp, ef, vz);
-                    if (!(coll && S.leapfrog)) vz = fma_(Ksp, ef, vz);
-                    int cn;
-                    T fn;
-                    const int side = drift(N, dtdx, c, f, vz, cn, fn, err);
-                    if (side < 0) {
-                        P0 = Part<T>{cn, fn, vx, vy, vz};
-                        alive = true;
-                    } else {
-                        atomicAdd(&s_cnt[CNT_ABS + 2 * SP + side], 1u);
-                        if (SP == 1 && S.has_see)
-                            see = emit_see<T>(S, (uint32_t)base + i, step, seed, side, Pse, s_cnt);
+                    if (m1 | m2) {
+                        if (o & 2u) move_rec<T>(S.sc, S.sp_, obase + q, offS + __popc(m1 & lt));
+                        if (o & 4u) move_rec<T>(S.bc, S.bp, obase + q, offB + __popc(m2 & lt));
+                        offS += __popc(m1);
+                        offB += __popc(m2);
+                        __syncwarp();
                     }
                 }
-                warp_dep(s_dep, alive ? P0.c : -1, alive ? cic_F(P0.f) : 0ull, lane);
+            }
+            if (qn) __syncwarp();
+            // ---- all particles: gather, half kicks, energy moment, drift, walls, deposit, survivors
+            const T dtdx = S.k.dtdx, kE = S.k.kappa_E;
+            int32_t* __restrict__ cout = S.c[1 - in_buf];
+            void* pout = S.p[1 - in_buf];
+            int c_next = scell[lane];
+            R r_next = srec[lane];
+#pragma unroll 1
+            for (int k = 0; k < PPT; ++k) {
+                if (32 * k >= cnt) break;
+                const int i = 32 * k + lane, craw = c_next;
+                const R r = r_next;
+                if (k + 1 < PPT) {  // the next row's loads, before this row's atomics
+                    c_next = scell[i + 32];
+                    r_next = srec[i + 32];
+                }
+                // branch-free for the common case: a lane without a particle computes on cell 0 and
+                // takes no part in the atomics and stores; rare cases behind warp votes
+                const bool coll = (craw & COLLIDED) != 0, in = i < cnt;
+                const int c0 = craw & ~COLLIDED;
+                const bool valid = in && (unsigned)c0 < (unsigned)N;
+                const int c = valid ? c0 : 0;
+                const T2 e = s_E[c];
+                const T ef = fma_(r.x, e.y, e.x);
+                const T vzn = fma_(Ksp, ef, r.w);  // v_n
+                if (SP == 0)
+                    energy_add<T>(h, S.Qg, valid && !coll, c, r.x, fma_(r.y, r.y, fma_(r.z, r.z, mul_(vzn, vzn))), kE,
+                                  lane);
+                const T vz = coll ? r.w : fma_(Ksp, ef, vzn);
+                int cn;
+                T fn, s;
+                const bool alive = drift_fast(N, dtdx, c, r.x, vz, cn, fn, s) && valid;
                 const unsigned mA = __ballot_sync(FULL, alive);
-                if (alive) store_rec<T>(cout, pout, offA + __popc(mA & lt), P0);
+                bool see = false;
+                Part<T> Pse{};
+                if (__any_sync(FULL, in && !alive) && in && !alive) {
+                    if (!valid || !(s == s)) err |= ERR_NONFINITE;  // a corrupt cell index is dropped too
+                    if (valid) {
+                        const int side = s >= (T)0 ? 1 : 0;
+                        atomicAdd(&s_cnt[CNT_ABS + 2 * SP + side], 1u);
+                        if (SP == 1 && S.has_see)
+                            see = emit_see<T>(S, S.Dother + s_dpar * (N + 1), (uint32_t)base + i, rs, side, Pse, s_cnt);
+                    }
+                }
+                warp_dep<SP == 1>(h, alive ? cn : -1, cic_F(fn), lane);
+                if (alive) store_rec<T>(cout, pout, offA + __popc(mA & lt), Part<T>{cn, fn, r.y, r.z, vz});
                 offA += __popc(mA);
-                if (SP == 1) {
+                if (SP == 1 && S.has_see) {
                     const unsigned mB = __ballot_sync(FULL, see);
                     if (see) store_rec<T>(S.bc, S.bp, offB + __popc(mB & lt), Pse);
                     offB += __popc(mB);
@@ -891,105 +972,115 @@ __global__ void __launch_bounds__(BLOCK, sweep_min_blocks<T, BLOCK, PPT>())
             S.cnt_main[cs] = (int)a;
             S.cnt_birth[cs] = (int)b;
             if (SP == 0) S.cnt_same[cs] = (int)c;
-            unsigned* sl = S.slice_tot + 3 * (cs / SLICE);
+            unsigned* sl = S.slice_tot + s_par * S.slice_stride + 3 * (cs / SLICE);
             if (a) atomicAdd(&sl[0], a);
             if (b) atomicAdd(&sl[1], b);
             if (SP == 0 && c) atomicAdd(&sl[2], c);
         }
     };
 
-    // tiles between flushes: at most 2^14 particles (and as many newborns) per flush, which keeps
-    // every histogram piece below 2^32
-    constexpr int FLUSH_TILES = (16384 / (BLOCK * PPT)) > 0 ? 16384 / (BLOCK * PPT) : 1;
-    int it = 0, since = 0;
-    for (int g = blockIdx.x; g < total_tiles; g += gridDim.x, ++it, ++since) {
-        // the store of tile g: the CTA's tiles increase, so its store only moves forward
-        int seg = cur_seg < 0 ? 0 : cur_seg;
-        while (seg + 1 < 2 * n_disc && s_segstart[seg + 1] <= g) ++seg;
-        if (seg == cur_seg && since >= FLUSH_TILES) {
-            flush();
-            since = 0;
-        }
-        if (seg != cur_seg) {
-            since = 0;
-            if (cur_seg >= 0) flush();
-            const int d = seg >> 1, sp = seg & 1;
-            if (tid == 0) {
-                const Disc& D = discs[d];
-                S.k = consts_of<T>(D);
-                S.d = d;
-                S.sp = sp;
-                S.N = D.N;
-                S.n_pts = D.n_pts;
-                S.has_see = D.has_see;
-                S.leapfrog = D.leapfrog;
-                S.n_exc = D.n_exc;
-                S.thr = D.thr[sp];
-                S.did = D.discharge_id;
-                S.n = s_store[seg].n;
-                S.cap = D.cap[sp];
-                S.bcap = D.bcap;
-                S.cin = D.c[in_buf][sp];
-                S.pin = D.p[in_buf][sp];
-                S.cout = D.c[1 - in_buf][sp];
-                S.pout = D.p[1 - in_buf][sp];
-                S.bc = D.bc[sp];
-                S.bp = D.bp[sp];
-                S.sc = D.sc;
-                S.sp_ = D.sp_;
-                S.Te = D.Te;
-                S.Ti = D.Ti;
-                S.Dg = D.D[sp];
-                S.Dother = D.D[1 - sp];
-                S.Qg = D.Q;
-                S.cnt = D.cnt;
-                S.start = D.start[sp];
-                S.K = s_store[seg].K;
-                S.M = s_store[seg].M;
-                S.D0 = s_store[seg].D0;
-                S.ralloc = D.ralloc[sp];
-                S.cnt_main = D.cnt_main[sp];
-                S.cnt_birth = D.cnt_birth[sp];
-                S.cnt_same = D.cnt_same;
-                S.slice_tot = D.slice_tot[sp] + (size_t)s_par * 3 * D.slice_n[sp];
+    // Adds the CTA's histograms and counters to the global sums of the current discharge and clears them.
+    auto flush = [&](int sp_cur) {
+        __syncthreads();
+        const int N = s_seg[0].N;
+        const bool folds = s_w0[0] != NO_WIN || s_w0[1] != NO_WIN;
+        for (int k = tid; folds && k < sweep_hist_words(sets) * WIN; k += nthr) {  // fold and clear the windows
+            const int a = k / WIN, j = k % WIN, sp = sets == 2 ? a >= 5 : sp_cur;
+            uint4* w = reinterpret_cast<uint4*>(s_win + a * WWORDS + j * WCOP);  // all zero without a window
+            const uint4 x = w[0], y = w[1];
+            const unsigned v = x.x + x.y + x.z + x.w + y.x + y.y + y.z + y.w;
+            if (v) {
+                s_h[a * max_N + s_w0[sp] + j] += v;
+                w[0] = w[1] = make_uint4(0u, 0u, 0u, 0u);
             }
-            if (tid < NCNT) s_cnt[tid] = 0;
-            __syncthreads();
-            for (int j = tid; j < h32_words; j += BLOCK) s_h32[j] = 0;
-            if (d != cur_d) {
-                const T* E = reinterpret_cast<const T*>(discs[d].E);
-                for (int j = tid; j <= S.N; j += BLOCK) s_E[j] = E[j];
-                cur_d = d;
-            }
-            cur_seg = seg;
-            __syncthreads();
         }
+        if (folds) __syncthreads();
+        for (int sp = 0; sp < 2; ++sp) {
+            if (sets == 1 && sp != sp_cur) continue;
+            unsigned* h = s_h + (sp == 1 && sets == 2 ? 5 * max_N : 0);
+            unsigned long long* Dg = s_seg[sp].Dg + s_dpar * (N + 1);
+            for (int j = tid; j <= N; j += nthr) {
+                unsigned long long v = 0, q = 0;
+                if (j < N) {
+                    v = ((unsigned long long)h[j] << 32) -
+                        ((unsigned long long)h[j + max_N] + ((unsigned long long)h[j + 2 * max_N] << 16));
+                    if (sp == 0) q = (unsigned long long)h[j + 3 * max_N] - h[j + 4 * max_N];
+                }
+                if (j > 0) {
+                    v += (unsigned long long)h[j - 1 + max_N] + ((unsigned long long)h[j - 1 + 2 * max_N] << 16);
+                    if (sp == 0) q += h[j - 1 + 4 * max_N];
+                }
+                if (v) atomicAdd(&Dg[j], v);
+                if (sp == 0 && q) atomicAdd(&s_seg[0].Qg[j], q);
+            }
+        }
+        if (tid < NCNT && s_cnt[tid]) atomicAdd(&s_seg[0].cnt[tid], (unsigned long long)s_cnt[tid]);
+    };
+    auto clear = [&]() {
+        __syncthreads();
+        for (int j = tid; j < sweep_hist_words(sets) * max_N; j += nthr) s_h[j] = 0;  // the windows: in the flush
+        if (tid < NCNT) s_cnt[tid] = 0;
+        __syncthreads();
+    };
 
-        const int b = it & 1;
-        const bool mine = pf[3] != 0;
-        const unsigned cs = (unsigned)pf[0];
-        const int base = pf[1], end = pf[2];
-        if (mine) {  // this tile's chunk: its staged data, then the next tile's prefetch into the other buffer
-            if (!mbar_wait(&s_mbar[warp][b], ((unsigned)pf[5] >> b) & 1u)) err |= ERR_TIMEOUT;
+    const int flush_rounds = max(1, flush_particles<T>() / (NW * CHUNK));
+    int cur_d = -1, cur_sp = 0;
+    for (int s = next_store(-1); s < n_store; s = next_store(s)) {
+        const int d = s >> 1, sp = s & 1;
+        if (cur_d >= 0 && (d != cur_d || sets == 1)) {
+            flush(cur_sp);
+            clear();
         }
-        __syncwarp();
-        if (lane == 0 && mine) pf[5] ^= 1 << b;
-        prefetch(b ^ 1, g + gridDim.x);
-        __syncwarp();
-        if (mine && !(err & ERR_TIMEOUT)) {
-            unsigned char* buf = stage + (size_t)b * sweep_stage_bytes<T, PPT>();
-            R* srec = reinterpret_cast<R*>(buf);
-            const int32_t* scell = reinterpret_cast<const int32_t*>(buf + REC_BYTES);
-            // slots and record offsets fit in 31 bits: the host caps every record buffer below 2^31
-            if (S.sp == 0) chunk(cs, base, end - base, srec, scell, IC<0>{});
-            else chunk(cs, base, end - base, srec, scell, IC<1>{});
+        if (d != cur_d) {
+            if (n_disc > 1) {
+                load_seg(d);
+                __syncthreads();
+            }
+            const int N = s_seg[0].N;
+            if (lane == 0 && warp < 2) {  // the species' window: around the first cells of the CTA's first and
+                const int q = warp;       // last chunk (any value is right)
+                const int2 g = s_range[2 * d + q];
+                int w0 = NO_WIN;
+                if (g.y - g.x >= WIN_CHUNKS) {
+                    const StoreSnap ss = s_store[2 * d + q];
+                    auto first_cell = [&](int k) {
+                        return __ldcg(s_seg[q].c[in_buf] +
+                                      (k < ss.K ? (unsigned)k * CHUNK : (unsigned)(ss.D0 + (k - ss.K) * CHUNK)));
+                    };
+                    const int a = first_cell(g.x), b = first_cell(g.y - 1);
+                    w0 = max(0, min((min(max(a, 0), N) + min(max(b, 0), N)) / 2 - WIN / 2, N - WIN));
+                }
+                s_w0[q] = w0;
+            }
+            if (n_disc > 1) load_field();
+            __syncthreads();
+            cur_d = d;
         }
-        __syncwarp();
+        cur_sp = sp;
+        carry_q = 0xFFFFFFFFu;
+        const int rounds = (s_range[s].y - s_range[s].x + NW - 1) / NW;  // chunks of this store a warp has at most
+        for (int r = 0; r < rounds; ++r) {
+            if (r > 0 && r % flush_rounds == 0) {
+                flush(cur_sp);
+                clear();
+            }
+            if (pf_s != s) continue;
+            const unsigned cs = (unsigned)pf_k;
+            const int base = pf_base, cnt = pf_stop - pf_base, b = pf_b;
+            if (!mbar_wait(&s_mbar[warp][b], (phases >> b) & 1u)) err |= ERR_TIMEOUT;
+            phases ^= 1u << b;
+            __syncwarp();
+            prefetch_next();  // the warp's next chunk, into the other buffer
+            if (!(err & ERR_TIMEOUT)) {
+                unsigned char* buf = stage + (unsigned)b * sweep_stage_bytes<T, PPT>();
+                R* srec = reinterpret_cast<R*>(buf);
+                int32_t* scell = reinterpret_cast<int32_t*>(buf + REC_BYTES);
+                if (sp == 0) chunk(cs, base, cnt, srec, scell, IC<0>{}); else chunk(cs, base, cnt, srec, scell, IC<1>{});
+            }
+            __syncwarp();
+        }
     }
-    // copies still in flight (a prefetch is issued only for a tile this CTA takes, so none should
-    // be): wait for them, bounded, before the CTA's shared memory goes away
-    if (pf[3] && !mbar_wait(&s_mbar[warp][it & 1], ((unsigned)pf[5] >> (it & 1)) & 1u)) err |= ERR_TIMEOUT;
-    if (cur_seg >= 0) flush();
+    if (cur_d >= 0) flush(cur_sp);
     if (err) atomicOr(&s_err, err);
     __syncthreads();
     if (tid == 0 && s_err) atomicOr(&ctl->error, s_err);
@@ -997,91 +1088,50 @@ __global__ void __launch_bounds__(BLOCK, sweep_min_blocks<T, BLOCK, PPT>())
 
 
 // ---------------------------------------------------------------------------
-// Exact prefix terms of the Poisson solve for both species over a run of nodes: r = sum of the
-// deposits D_k, m = sum of k D_k. With R_j = sum_{1<=k<=j} D_k and M_j = sum_{1<=k<=j} k D_k the
-// double sum S_{j+1} = sum_{i<=j} R_i equals (j + 1) R_j - M_j, so one scan of plain integer sums
-// gives both R and S (no products inside the scan; integer, so any order gives the same).
+// Exact prefix terms of the Poisson solve over a run of nodes, per species: r = sum of the deposits
+// D_k, and the sum of k D_k in two 64-bit halves, a of the low and b of the high 32 bits of D_k (so no
+// sum needs a carry chain). With R_j = sum_{1<=k<=j} D_k and M_j = sum_{1<=k<=j} k D_k = b 2^32 + a the
+// double sum S_{j+1} = sum_{i<=j} R_i equals (j + 1) R_j - M_j, so one scan of plain integer sums gives
+// both R and S (integer, so any order gives the same).
 struct PSum {
-    unsigned long long r[2];
-    unsigned __int128 m[2];
+    unsigned long long v[6];  // r of electrons, ions; a; b
+    __device__ __forceinline__ void add(int j, unsigned long long de, unsigned long long di) {
+        v[0] += de;
+        v[1] += di;
+        v[2] += (unsigned long long)j * (unsigned)de;
+        v[3] += (unsigned long long)j * (unsigned)di;
+        v[4] += (unsigned long long)j * (unsigned)(de >> 32);
+        v[5] += (unsigned long long)j * (unsigned)(di >> 32);
+    }
 };
-__device__ __forceinline__ void psum_add(PSum& a, const PSum& b) {
-#pragma unroll
-    for (int sp = 0; sp < 2; ++sp) {
-        a.r[sp] += b.r[sp];
-        a.m[sp] += b.m[sp];
-    }
-}
-__device__ __forceinline__ PSum psum_shfl_up(const PSum& x, int o) {
-    PSum y;
-#pragma unroll
-    for (int sp = 0; sp < 2; ++sp) {
-        y.r[sp] = __shfl_up_sync(FULL, x.r[sp], o);
-        const unsigned long long lo = __shfl_up_sync(FULL, (unsigned long long)x.m[sp], o);
-        const unsigned long long hi = __shfl_up_sync(FULL, (unsigned long long)(x.m[sp] >> 64), o);
-        y.m[sp] = ((unsigned __int128)hi << 64) | lo;
-    }
-    return y;
-}
-// Exclusive scan of one PSum per thread over the first NT threads of the block (NT / 32 warps,
-// named barrier 1; the other warps of the block do not take part), and the total over all of
-// them. s_w: NT / 32 + 1 entries.
-template <int NT>
-__device__ __forceinline__ PSum block_exclusive_psum(const PSum& own, PSum* s_w, int lane, int warp, PSum& total) {
-    constexpr int NW = NT / 32;
-    PSum x = own;
-#pragma unroll 1
-    for (int o = 1; o < 32; o <<= 1) {
-        const PSum y = psum_shfl_up(x, o);
-        if (lane >= o) psum_add(x, y);
-    }
-    if (lane == 31) s_w[warp] = x;
-    asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
-    if (warp == 0) {
-        const PSum v = lane < NW ? s_w[lane] : PSum{};
-        PSum w = v;
-#pragma unroll 1
-        for (int o = 1; o < NW; o <<= 1) {
-            const PSum y = psum_shfl_up(w, o);
-            if (lane >= o) psum_add(w, y);
-        }
-        if (lane == NW - 1) s_w[NW] = w;
-        if (lane < NW) {
-#pragma unroll
-            for (int sp = 0; sp < 2; ++sp) {  // inclusive -> exclusive
-                w.r[sp] -= v.r[sp];
-                w.m[sp] -= v.m[sp];
-            }
-            s_w[lane] = w;
-        }
-    }
-    asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
-    total = s_w[NW];
-    PSum r = s_w[warp];
-#pragma unroll
-    for (int sp = 0; sp < 2; ++sp) {  // + this warp's inclusive sum before the thread
-        r.r[sp] += x.r[sp] - own.r[sp];
-        r.m[sp] += x.m[sp] - own.m[sp];
-    }
-    return r;
-}
 // Nearest double of a 128-bit integer below 2^115 in magnitude (two roundings at most).
 __device__ __forceinline__ double i128_to_double(__int128 x) {
     const long long hi = (long long)(x >> 64);
     const unsigned long long lo = (unsigned long long)x;
     return __fma_rn((double)hi, 0x1p64, __ull2double_rn(lo));
 }
-
-// After a sweep (mode bit 1) and for every solve, one grid (x = slice or role,
-// y = store): CTAs x < nsl write the region starts of the chunks of slice x of
-// store y (the first slot each chunk's survivors take in the new layout) and
-// copy its newborns into the newborn area; CTA x = nsl, y even solves the field
-// of discharge y / 2 and accumulates the moments; CTA x = nsl, y odd turns the
-// slice sums of discharge y / 2 into the new counts and layouts and clears the
-// sums of the other parity for the next sweep. mode bits: 1 layouts after a sweep; 2
-// accumulate moments and advance the step; 4 initial solve at t = n dt (load);
-// 8 segments only (no solve, deposits kept). The last CTA to finish advances
-// the step (mode bit 2) and flips the slice parity (mode bit 1).
+// S at node j1 from the sums through node j1 - 1, in charge units: pr1 S_ions - pr0 S_electrons. Out of
+// line: the grid runs once per step from a cold instruction cache, where a second copy costs more than
+// the call.
+__device__ __noinline__ double poisson_S(unsigned long long r0, unsigned long long r1, unsigned long long a0,
+                                         unsigned long long a1, unsigned long long b0, unsigned long long b1, int j1,
+                                         double pr0, double pr1) {
+    const __int128 S0 = (__int128)((unsigned __int128)(unsigned)j1 * r0 - (((unsigned __int128)b0 << 32) + a0));
+    const __int128 S1 = (__int128)((unsigned __int128)(unsigned)j1 * r1 - (((unsigned __int128)b1 << 32) + a1));
+    return __fma_rn(pr1, i128_to_double(S1), -pr0 * i128_to_double(S0));
+}
+// After a sweep (mode bit 1) and for every solve, one grid (x = slice or role, y = store):
+//   x < nsl          the region starts of the chunks of slice x of store y (the first slot each chunk's
+//                    survivors take in the new layout) and its newborns, copied into the newborn area;
+//   y even, x >= nsl the field of discharge y / 2 at the FIELD_NODES nodes of part x - nsl (every part
+//                    scans all deposits; the FP64 work per node, slow on this part, is what is split);
+//   y odd, x == nsl  the slice sums of discharge y / 2 into the new counts and layouts, the sums of the
+//                    other parity cleared for the next sweep;
+//   y odd, x > nsl   the moments of the nodes of part x - nsl - 1, and the deposits of the previous
+//                    solve (the other deposit parity) cleared for the next sweep.
+// mode bits: 1 layouts after a sweep; 2 accumulate moments and advance the step; 4 initial solve at t =
+// n dt (load); 8 segments only (no solve, deposits kept). The last CTA to finish advances the step (mode
+// bit 2) and flips the slice parity (mode bit 1) and the deposit parity (a solve).
 template <int BLOCK>
 __device__ __forceinline__ void seg_apply(const Disc* __restrict__ discs, Ctl* __restrict__ ctl, int out_buf, int tid, int lane,
                           int warp) {
@@ -1126,14 +1176,14 @@ __device__ __forceinline__ void seg_apply(const Disc* __restrict__ discs, Ctl* _
         const unsigned* Tp = slice_s + (size_t)par * 3 * sn_s;
         long long a = 0, b = 0, c = 0;
         for (int k = lane; k < (int)blockIdx.x; k += 32) {
-            a += Tp[3 * k + 0];
-            b += Tp[3 * k + 1];
-            c += Tp[3 * k + 2];
+            a += __ldcg(Tp + 3 * k + 0);
+            b += __ldcg(Tp + 3 * k + 1);
+            c += __ldcg(Tp + 3 * k + 2);
         }
         if (sp == 1) {
             const long long ch0 = ctl->chunks_in[d][0];
             const unsigned* T0 = slice0 + (size_t)par * 3 * sn0;
-            for (long long k = lane; k < (ch0 + SLICE - 1) / SLICE; k += 32) b += T0[3 * k + 2];
+            for (long long k = lane; k < (ch0 + SLICE - 1) / SLICE; k += 32) b += __ldcg(T0 + 3 * k + 2);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -1151,9 +1201,9 @@ __device__ __forceinline__ void seg_apply(const Disc* __restrict__ discs, Ctl* _
     for (int i = 0; i < K; ++i) {
         const int k = i * BLOCK + tid;
         const bool in = t0 + k < chunks;
-        s_cnt[0][k] = (unsigned short)(in ? cnt_m[t0 + k] : 0);
-        s_cnt[1][k] = (unsigned short)(in ? cnt_b[t0 + k] : 0);
-        s_cnt[2][k] = (unsigned short)((in && sp == 0) ? cnt_s[t0 + k] : 0);
+        s_cnt[0][k] = (unsigned short)(in ? __ldcg(cnt_m + t0 + k) : 0);
+        s_cnt[1][k] = (unsigned short)(in ? __ldcg(cnt_b + t0 + k) : 0);
+        s_cnt[2][k] = (unsigned short)((in && sp == 0) ? __ldcg(cnt_s + t0 + k) : 0);
     }
     __syncthreads();
     const long long tb = t0 + (long long)tid * K;
@@ -1231,9 +1281,9 @@ __device__ __forceinline__ void seg_apply(const Disc* __restrict__ discs, Ctl* _
             while (ci < K - 1 && rem >= s_cnt[row][tw + ci]) rem -= s_cnt[row][tw + ci++];
             const long long srcr = (t0 + tw + ci) * CHUNK + rem;
             if (j < bcap) {  // records of one (FP32) or two (FP64) 16-byte words; no runtime-indexed array
-                const int cv = cin[srcr];
-                const R r0 = pin[srcr * rw];
-                const R r1 = rw == 2 ? pin[srcr * rw + 1] : r0;
+                const int cv = __ldcg(cin + srcr);
+                const R r0 = __ldcg(pin + srcr * rw);
+                const R r1 = rw == 2 ? __ldcg(pin + srcr * rw + 1) : r0;
                 cdst[j] = cv;
                 pdst[j * rw] = r0;
                 if (rw == 2) pdst[j * rw + 1] = r1;
@@ -1245,216 +1295,259 @@ __device__ __forceinline__ void seg_apply(const Disc* __restrict__ discs, Ctl* _
     if (err) atomicOr(&ctl->error, err);
 }
 
-// Field of one discharge after its deposits are complete (the field role of k_post; all
-// POST_BLOCK threads of the CTA). Poisson, Eq. (poisson): phi_{j-1} - 2 phi_j + phi_{j+1} = -r_j with
-// r_j = rho_j dx^2 / eps0, phi_0 = V_rf sin(2 pi f t), phi_N = 0. With R_j = sum_{k<=j} r_k and
-// S_j = sum_{i<j} R_i: phi_j = phi_0 + j g_1 - S_j, g_1 = (phi_N - phi_0 + S_N) / N. R and S are
-// linear in the deposits: R_j = c_i IR_i,j - c_e IR_e,j, S_{j+1} = c_i IS_i,j - c_e IS_e,j with the
-// exact integer sums IR_s,j = sum_{1<=k<=j} D_s,k (64 bits: a store holds below 2^30 particles of
-// 2^32 each) and IS_s,j = sum_{i<=j} IR_s,i (128 bits), from one scan of plain sums (PSum). FP64
-// (slow on this part) is used once per node, with no division (host reciprocals).
-constexpr int POST_BLOCK = 512;  // threads per k_post CTA
-constexpr int FIELD_SCAN = 256;  // threads of the integer scan
+constexpr int POST_BLOCK = 512;   // threads per k_post CTA
+constexpr int FIELD_NODES = 128;  // nodes of a field or moments part
+constexpr int FIELD_SUMS = 128;   // partial sums of the solve
 
 // Discharge current density over step n (section "Boundary conditions", equation for J(t)):
 // J = eps0 dE/dt + e0 (Gamma_i - Gamma_e), with the particle fluxes counted positive towards +z
 // from the step's absorbed and emitted superparticles: at z = 0 an absorbed ion (moving towards
 // -z) carries -e w_i, an absorbed electron +e w_e, an emitted secondary electron (towards +z)
 // -e w_e; at z = d the absorbed particles' signs flip and emitted electrons move towards -z.
-// FP64, by one thread of the field CTA after the new electrode fields Ew are known. The initial
-// solve of a load (mode bit 4) only records the fields and counters. On a full step the current at
-// z = 0 is also projected onto the rf period's first harmonic (sin and cos at the step midpoint);
-// at the end of a period the amplitude is stored.
-__device__ __forceinline__ void discharge_current(const Disc& D, int d, Ctl* ctl, int mode, long long step,
-                                               const double* Ew) {
-    // counters as scalars (an array here would live in local memory, cold at every step)
-    const unsigned long long c0 = D.cnt[CNT_ABS + 0], c1 = D.cnt[CNT_ABS + 1], c2 = D.cnt[CNT_ABS + 2],
-                             c3 = D.cnt[CNT_ABS + 3];  // [species][electrode]
-    const unsigned long long c4 = D.cnt[CNT_SEE_SIDE], c5 = D.cnt[CNT_SEE_SIDE + 1];
-    if (!(mode & 4)) {  // a solve after a sweep (or a stand-alone solve): the current of step n
-        double J0 = 0.0, JN = 0.0;  // no earlier solve: no current
-        if (ctl->have_solve[d]) {
-            const unsigned long long* cs = ctl->cnt_solve[d];
-            const double dA0 = (double)(c0 - cs[0]), dA1 = (double)(c1 - cs[1]), dA2 = (double)(c2 - cs[2]),
-                         dA3 = (double)(c3 - cs[3]);
-            const double dS0 = (double)(c4 - cs[4]), dS1 = (double)(c5 - cs[5]);
-            const double we = D.w[0], wi = D.w[1], rdt = D.inv_dt;  // FP64 division is slow on this part
-            const double cond0 = E_CHARGE * (we * dA0 - wi * dA2 - we * dS0) * rdt;
-            const double condN = E_CHARGE * (wi * dA3 - we * dA1 + we * dS1) * rdt;
-            J0 = EPS0 * (Ew[0] - ctl->E_wall[d][0]) * rdt + cond0;
-            JN = EPS0 * (Ew[1] - ctl->E_wall[d][1]) * rdt + condN;
+// FP64, by one thread of the first field part beside the node field: everything that does not need
+// the new electrode fields is read and formed before they are known (before()). The initial solve of a
+// load (mode bit 4) only records the fields and counters. On a full step the current at z = 0 is also
+// projected onto the rf period's first harmonic (sin and cos at the step midpoint); at the end of a
+// period the amplitude is stored.
+struct Current {
+    unsigned long long c[6];
+    double cond0, condN, E0, EN, js0, js1, jt0, jt1, vs;
+    int have, k, jslot, par;
+    __device__ __forceinline__ void before(const Disc& D, int d, const Ctl* ctl, long long step) {
+        unsigned long long o[6];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) c[i] = __ldcg(D.cnt + CNT_ABS + i);  // [species][electrode]
+        c[4] = __ldcg(D.cnt + CNT_SEE_SIDE);
+        c[5] = __ldcg(D.cnt + CNT_SEE_SIDE + 1);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) o[i] = ctl->cnt_solve[d][i];
+        have = ctl->have_solve[d];
+        E0 = ctl->E_wall[d][0];
+        EN = ctl->E_wall[d][1];
+        js0 = ctl->J_sum[d][0];
+        js1 = ctl->J_sum[d][1];
+        par = ctl->dep_par;
+        vs = ctl->V_scale[d][par];
+        jslot = step_mod(step, D.jh);
+        k = 0;
+        if (D.jtab) {
+            k = step_mod(step, D.steps_per_period);
+            jt0 = D.jtab[2 * k];
+            jt1 = D.jtab[2 * k + 1];
         }
-        const long long slot = step % D.jh;
-        D.J_hist[2 * slot] = J0;
-        D.J_hist[2 * slot + 1] = JN;
-        if ((mode & 2) && D.jtab && D.steps_per_period > 0) {
+        const double we = D.w[0], wi = D.w[1], rdt = D.inv_dt;  // FP64 division is slow on this part
+        cond0 = E_CHARGE * (we * (double)(c[0] - o[0]) - wi * (double)(c[2] - o[2]) - we * (double)(c[4] - o[4])) * rdt;
+        condN = E_CHARGE * (wi * (double)(c[3] - o[3]) - we * (double)(c[1] - o[1]) + we * (double)(c[5] - o[5])) * rdt;
+    }
+    __device__ __forceinline__ void after(const Disc& D, int d, Ctl* ctl, int mode, long long step, double Ew0,
+                                          double Ew1) {
+        ctl->E0_last[d] = Ew0;
+        if (!(mode & 4)) {  // a solve after a sweep (or a stand-alone solve): the current of step n
+            const double rdt = D.inv_dt;
+            double J0 = 0.0, JN = 0.0;  // no earlier solve: no current
+            if (have) {
+                J0 = EPS0 * (Ew0 - E0) * rdt + cond0;
+                JN = EPS0 * (Ew1 - EN) * rdt + condN;
+            }
+            D.J_hist[2 * jslot] = J0;
+            D.J_hist[2 * jslot + 1] = JN;
             const int spp = D.steps_per_period;
-            const int k = (int)(step % spp);
-            ctl->J_sum[d][0] += J0 * D.jtab[2 * k];
-            ctl->J_sum[d][1] += J0 * D.jtab[2 * k + 1];
-            if (k == spp - 1) {
-                const double a = 2.0 * ctl->J_sum[d][0] / spp, b = 2.0 * ctl->J_sum[d][1] / spp;
-                const double amp = sqrt(a * a + b * b);
-                D.J_amp[(step / spp) % PERIOD_HIST] = amp;
-                D.V_hist[(step / spp) % PERIOD_HIST] = D.V_rf * ctl->V_scale[d];
-                const double J0 = ctl->J_drive[d];
-                if (J0 > 0.0 && amp > 0.0) ctl->V_scale[d] = ctl->V_scale[d] * (J0 / amp);  // Eq. (adaptivevoltage)
-                ctl->J_sum[d][0] = 0.0;
-                ctl->J_sum[d][1] = 0.0;
+            if ((mode & 2) && D.jtab && spp > 0) {
+                js0 += J0 * jt0;
+                js1 += J0 * jt1;
+                if (k == spp - 1) {
+                    const double a = 2.0 * js0 / spp, b = 2.0 * js1 / spp;
+                    const double amp = sqrt(a * a + b * b);
+                    const long long per = step_div(step, spp) % PERIOD_HIST;
+                    D.J_amp[per] = amp;
+                    D.V_hist[per] = D.V_rf * vs;
+                    const double Jd = ctl->J_drive[d];
+                    if (Jd > 0.0 && amp > 0.0) vs = vs * (Jd / amp);  // Eq. (adaptivevoltage)
+                    js0 = js1 = 0.0;
+                }
+                ctl->J_sum[d][0] = js0;
+                ctl->J_sum[d][1] = js1;
             }
         }
+        ctl->V_scale[d][par ^ 1] = vs;  // for the next solve (other parts may still read this one's)
+        ctl->have_solve[d] = 1;
+        ctl->E_wall[d][0] = Ew0;
+        ctl->E_wall[d][1] = Ew1;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) ctl->cnt_solve[d][i] = c[i];
     }
-    ctl->have_solve[d] = 1;
-    ctl->E_wall[d][0] = Ew[0];
-    ctl->E_wall[d][1] = Ew[1];
-    unsigned long long* cs = ctl->cnt_solve[d];
-    cs[0] = c0;
-    cs[1] = c1;
-    cs[2] = c2;
-    cs[3] = c3;
-    cs[4] = c4;
-    cs[5] = c5;
-}
+};
+
+// Field of one discharge after its deposits are complete, nodes of part `part`. Poisson, Eq. (poisson):
+// phi_{j-1} - 2 phi_j + phi_{j+1} = -r_j with r_j = rho_j dx^2 / eps0, phi_0 = V_rf sin(2 pi f t),
+// phi_N = 0. With R_j = sum_{k<=j} r_k and S_j = sum_{i<j} R_i: phi_j = phi_0 + j g_1 - S_j, g_1 = (phi_N
+// - phi_0 + S_N) / N. R and S are linear in the deposits: R_j = c_i IR_i,j - c_e IR_e,j, S_{j+1} = c_i
+// IS_i,j - c_e IS_e,j with the exact integer sums IR_s,j = sum_{1<=k<=j} D_s,k (64 bits: a store holds
+// below 2^30 particles of 2^32 each) and IS_s,j = sum_{i<=j} IR_s,i (128 bits), from one scan (PSum).
+//
+// What bounds it is latency, above all instruction fetches: the grid runs once per step after other
+// code, so the code is short: one small scan run by six warps, one sum each (the earlier scan held
+// 128-bit pairs in registers), J(t) in a warp of its own, loads requested together. FP64 (2 operations per
+// clock and SM here) is used once per node, with no division (host reciprocals), 128 nodes to a CTA: at
+// 2048 cells one CTA took 14 us for all of them. Measured, a launch: 13.1 -> 8.5 us at 128 cells, 18.9 ->
+// 8.9 at 512, 30.1 -> 12.9 at 2048, 21.8 -> 13.1 for 16 discharges.
 template <typename T>
-__device__ __forceinline__ void field_solve(const Disc& D, int d, Ctl* __restrict__ ctl, int mode, int tid, int lane,
-                                            int warp, double* s_f, int max_N, PSum* s_ps, double* s_Ew) {
-    constexpr int BLOCK = POST_BLOCK;
-    // every field of the discharge is read before the first store
+__device__ __forceinline__ void field_solve(const Disc& D, int d, Ctl* __restrict__ ctl, int mode, int part, int tid,
+                                            int lane, int warp, unsigned long long* s_f, int max_N,
+                                            unsigned long long (*s_ps)[FIELD_SUMS], unsigned long long* s_tot,
+                                            double* s_g1, Current& J) {
     const int N = D.N;
-    unsigned long long* __restrict__ De = D.D[0];
-    unsigned long long* __restrict__ Di = D.D[1];
-    unsigned long long* __restrict__ Qd = D.Q;
-    unsigned long long* __restrict__ Dp = D.Dprev;
-    unsigned __int128* __restrict__ aDe = D.acc_D[0];
-    unsigned __int128* __restrict__ aDi = D.acc_D[1];
-    unsigned __int128* __restrict__ aQ = D.acc_Q;
-    unsigned __int128* __restrict__ aDp = D.acc_Dprev;
-    double* __restrict__ phi = D.phi;
-    double* __restrict__ E64 = D.E64;
-    T* __restrict__ Ef = reinterpret_cast<T*>(D.E);
-    const double pr0 = D.pc_r[0], pr1 = D.pc_r[1], pw0 = D.pc_w[0], pw1 = D.pc_w[1];
-    const double inv_dx = D.inv_dx, m_inv_2dx = D.m_inv_2dx, hdx_eps = D.hdx_eps, inv_N = D.inv_N;
+    if (part * FIELD_NODES > N) return;
+    // everything that is read is requested first; the deposits of both parities, so that their loads need
+    // not wait for the parity
+    const int par = ctl->dep_par;
     const long long step = ctl->step;
-    const long long ns = (mode & 4) ? step : step + 1;  // time level of the solve
-    const double V0 = (D.V0tab ? D.V0tab[ns % D.steps_per_period]
-                               : D.V_rf * sin(2.0 * PI_D * D.f_rf * ((double)ns * D.dt))) *
-                      ctl->V_scale[d];
-    // one pass over the nodes: stage the deposits in shared memory, accumulate the moments (mode
-    // bit 2) and hand the next sweep zeroed deposit arrays
-    unsigned long long* sde = reinterpret_cast<unsigned long long*>(s_f);
+    const double vs0 = ctl->V_scale[d][0], vs1 = ctl->V_scale[d][1];
+    const bool cur = part == 0 && warp == POST_BLOCK / 32 - 1;  // the warp of J(t) (one thread of it)
+    unsigned long long* sde = s_f;
     unsigned long long* sdi = sde + (max_N + 1);
-    for (int j = tid; j <= N; j += BLOCK) {
-        const unsigned long long de = De[j], di = Di[j], q = Qd[j], dp = Dp[j];
-        if (mode & 2) {
-            const unsigned __int128 a0 = aDe[j], a1 = aDi[j], aq = aQ[j], ap = aDp[j];
-            aDe[j] = a0 + de;
-            aDi[j] = a1 + di;
-            aQ[j] = aq + q;
-            aDp[j] = ap + dp;
-        }
-        Dp[j] = de;
-        De[j] = 0;
-        Di[j] = 0;
-        Qd[j] = 0;
-        sde[j] = de;
-        sdi[j] = di;
+    for (int j = tid; j <= N; j += POST_BLOCK) {
+        const unsigned long long e0 = __ldcg(D.D[0] + j), e1 = __ldcg(D.D[0] + N + 1 + j);
+        const unsigned long long i0 = __ldcg(D.D[1] + j), i1 = __ldcg(D.D[1] + N + 1 + j);
+        sde[j] = par ? e1 : e0;
+        sdi[j] = par ? i1 : i0;
     }
-    if (tid == 0 && (mode & 2)) ctl->acc_steps[d] += 1;
+    const long long ns = (mode & 4) ? step : step + 1;  // time level of the solve
+    const double* Vt = D.V0tab;
+    const double Vk = Vt ? Vt[step_mod(ns, D.steps_per_period)] : 0.0;
     __syncthreads();
-    if (tid >= FIELD_SCAN) return;
-    // thread t owns nodes [lo, hi); node 0 carries no deposit term; node N is done by the owner of N - 1
-    const int per = (N + FIELD_SCAN - 1) / FIELD_SCAN;
-    const int lo = min(N, tid * per), hi = min(N, lo + per);
-    PSum own{};
-    for (int j = max(lo, 1); j < hi; ++j) {
-        own.r[0] += sde[j];
-        own.r[1] += sdi[j];
-        own.m[0] += (unsigned __int128)j * sde[j];
-        own.m[1] += (unsigned __int128)j * sdi[j];
+    // thread t < FIELD_SUMS sums the nodes [t per, (t + 1) per) (node 0 carries no deposit term), 1 <= j < N
+    const int per = (N + FIELD_SUMS - 1) / FIELD_SUMS;
+    if (tid < FIELD_SUMS) {
+        PSum own{};
+#pragma unroll 1
+        for (int j = max(tid * per, 1); j < min(N, (tid + 1) * per); ++j) own.add(j, sde[j], sdi[j]);
+        // lane l of the scan below takes threads 4 l .. 4 l + 3
+#pragma unroll
+        for (int q = 0; q < 6; ++q) s_ps[q][(tid & 3) * 32 + (tid >> 2)] = own.v[q];
     }
-    PSum tot;
-    PSum run = block_exclusive_psum<FIELD_SCAN>(own, s_ps, lane, warp, tot);
-    // R_j -> r_j sums in FP64 (Rr), S_{j+1} = (j + 1) R_j - M_j -> FP64 (Sx), as c_i x_i - c_e x_e
-    auto Rr_of = [&](const PSum& p) {
-        return __fma_rn(pr1, (double)(long long)p.r[1], -pr0 * (double)(long long)p.r[0]);
+    __syncthreads();
+    if (warp < 6) {  // exclusive scan of sum `warp` over the partial sums
+        unsigned long long* p = s_ps[warp] + lane;
+        const unsigned long long x0 = p[0], x1 = p[32], x2 = p[64], x3 = p[96];
+        const unsigned long long x = x0 + x1 + x2 + x3;
+        unsigned long long y = x;
+#pragma unroll 1
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long z = __shfl_up_sync(FULL, y, o);
+            if (lane >= o) y += z;
+        }
+        if (lane == 31) s_tot[warp] = y;
+        y -= x;
+        p[0] = y;
+        p[32] = y + x0;
+        p[64] = y + x0 + x1;
+        p[96] = y + x0 + x1 + x2;
+    } else if (cur && lane == 0) {
+        J.before(D, d, ctl, step);
+    }
+    __syncthreads();
+    const double pr0 = D.pc_r[0], pr1 = D.pc_r[1];
+    // R_j -> r_j sums in FP64, as c_i x_i - c_e x_e
+    auto Rr_of = [&](unsigned long long r0, unsigned long long r1) {
+        return __fma_rn(pr1, (double)(long long)r1, -pr0 * (double)(long long)r0);
     };
-    auto Sx_of = [&](const PSum& p, int j1) {  // S at node j1 from the sums through node j1 - 1
-        const __int128 S0 = (__int128)((unsigned __int128)j1 * p.r[0] - p.m[0]);
-        const __int128 S1 = (__int128)((unsigned __int128)j1 * p.r[1] - p.m[1]);
-        return __fma_rn(pr1, i128_to_double(S1), -pr0 * i128_to_double(S0));
+    const double V0 = (Vt ? Vk : D.V_rf * sin(2.0 * PI_D * D.f_rf * ((double)ns * D.dt))) * (par ? vs1 : vs0);
+    // warps 0-3: R_{j-1}, R_j and S_j of node j; the last warp: g_1 (with S_N from the totals), while they
+    // do not need it yet
+    const int j = part * FIELD_NODES + tid;
+    const bool node = tid < FIELD_NODES && j <= N, inside = node && j > 0 && j < N;
+    double Rprev = 0.0, Rj = 0.0, Sj = 0.0;
+    if (inside) {
+        PSum run;
+        const int t = j / per;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) run.v[q] = s_ps[q][(t & 3) * 32 + (t >> 2)];
+#pragma unroll 1
+        for (int i = max(t * per, 1); i < j; ++i) run.add(i, sde[i], sdi[i]);
+        Rprev = Rr_of(run.v[0], run.v[1]);
+        Rj = Rr_of(run.v[0] + sde[j], run.v[1] + sdi[j]);
+        Sj = poisson_S(run.v[0], run.v[1], run.v[2], run.v[3], run.v[4], run.v[5], j, pr0, pr1);
+    } else if (tid == POST_BLOCK - 32) {
+        *s_g1 = (poisson_S(s_tot[0], s_tot[1], s_tot[2], s_tot[3], s_tot[4], s_tot[5], N, pr0, pr1) - V0) * D.inv_N;
+    }
+    __syncthreads();
+    const double g1 = *s_g1;
+    // Gauss's law over the half cells at the electrodes
+    auto wall = [&](int n) {
+        const double rw = __fma_rn(D.pc_w[1], (double)sdi[n], -D.pc_w[0] * (double)sde[n]);
+        return n == 0 ? -g1 * D.inv_dx - rw * D.hdx_eps
+                      : -(g1 - Rr_of(s_tot[0], s_tot[1])) * D.inv_dx + rw * D.hdx_eps;
     };
-    const double g1 = (Sx_of(tot, N) - V0) * inv_N;  // S_N from the totals
+    if (cur && lane == 0) J.after(D, d, ctl, mode, step, wall(0), wall(N));
+    if (!node) return;
     // g_j = phi_j - phi_{j-1} = g_1 - R_{j-1}; node field E_j = -(g_j + g_{j+1}) / (2 dx) inside
-    // (the central difference of phi, without the cancellation of large phi values), and Gauss's
-    // law over the half cells at the electrodes
-    double Rprev = Rr_of(run);      // R_{lo-1}
-    double Sprev = Sx_of(run, lo);  // S_lo
-    for (int j = lo; j < hi; ++j) {
-        if (j >= 1) {
-            const unsigned long long e = sde[j], i = sdi[j];
-            run.r[0] += e;
-            run.r[1] += i;
-            run.m[0] += (unsigned __int128)j * e;
-            run.m[1] += (unsigned __int128)j * i;
-        }
-        const double Rj = Rr_of(run);
-        double ph, E;
-        if (j == 0) {
-            ph = V0;
-            const double rw = __fma_rn(pw1, (double)sdi[0], -pw0 * (double)sde[0]);
-            E = -g1 * inv_dx - rw * hdx_eps;
-            ctl->E0_last[d] = E;
-            s_Ew[0] = E;
-        } else {
-            ph = V0 + (double)j * g1 - Sprev;
-            E = ((g1 - Rprev) + (g1 - Rj)) * m_inv_2dx;
-        }
-        phi[j] = ph;
-        E64[j] = E;
-        Ef[j] = (T)E;
-        Rprev = Rj;
-        Sprev = Sx_of(run, j + 1);
+    // (the central difference of phi, without the cancellation of large phi values)
+    const double E = inside ? ((g1 - Rprev) + (g1 - Rj)) * D.m_inv_2dx : wall(j);
+    reinterpret_cast<T*>(D.E)[j] = (T)E;
+    D.E64[j] = E;
+    D.phi[j] = inside ? V0 + (double)j * g1 - Sj : j == 0 ? V0 : 0.0;
+}
+
+// The moments of the nodes of a part (mode bit 2), and zeroed arrays for the next sweep: the energy
+// moment and the deposits of the other parity, which are those at x_n (of the previous solve).
+__device__ __forceinline__ void moments_part(const Disc& D, int d, Ctl* __restrict__ ctl, int mode, int part, int tid) {
+    const int N = D.N, j = part * FIELD_NODES + tid;
+    if (part == 0 && tid == 0 && (mode & 2)) ctl->acc_steps[d] += 1;
+    if (tid >= FIELD_NODES || j > N) return;
+    const int par = ctl->dep_par;
+    const size_t po = (size_t)par * (N + 1) + j, pn = (size_t)(par ^ 1) * (N + 1) + j;
+    unsigned long long* __restrict__ D0 = D.D[0];
+    unsigned long long* __restrict__ D1 = D.D[1];
+    unsigned long long* __restrict__ Qd = D.Q;
+    if (mode & 2) {
+        unsigned __int128* __restrict__ acc = D.acc_D[0] + j;  // n_e, n_i, energy, n_e at x_n, N + 1 apart
+        const int n1 = N + 1;
+        const unsigned long long de = __ldcg(D0 + po), di = __ldcg(D1 + po), q = __ldcg(Qd + j), dp = __ldcg(D0 + pn);
+        auto ld128 = [](const unsigned __int128* a) {
+            const ulonglong2 v = __ldcg(reinterpret_cast<const ulonglong2*>(a));
+            return ((unsigned __int128)v.y << 64) | v.x;
+        };
+        const unsigned __int128 a0 = ld128(acc), a1 = ld128(acc + n1), a2 = ld128(acc + 2 * n1), a3 = ld128(acc + 3 * n1);
+        acc[0] = a0 + de;
+        acc[n1] = a1 + di;
+        acc[2 * n1] = a2 + q;
+        acc[3 * n1] = a3 + dp;
     }
-    if (lo < hi && hi == N) {  // the electrode at x = L
-        const double rw = __fma_rn(pw1, (double)sdi[N], -pw0 * (double)sde[N]);
-        const double E = -(g1 - Rprev) * inv_dx + rw * hdx_eps;
-        phi[N] = 0.0;
-        E64[N] = E;
-        Ef[N] = (T)E;
-        s_Ew[1] = E;
-    }
-    asm volatile("bar.sync 1, %0;" ::"n"(FIELD_SCAN) : "memory");
-    if (tid == 0) discharge_current(D, d, ctl, mode, step, s_Ew);
+    D0[pn] = 0;
+    D1[pn] = 0;
+    Qd[j] = 0;
 }
 
 template <typename T>
-__global__ void __launch_bounds__(POST_BLOCK, 1) k_post(const Disc* __restrict__ discs, int n_disc, Ctl* __restrict__ ctl,
+__global__ void __launch_bounds__(POST_BLOCK, 2) k_post(const Disc* __restrict__ discs, int n_disc, Ctl* __restrict__ ctl,
                                                      int out_buf, int mode, int nsl, int max_N) {
     constexpr int BLOCK = POST_BLOCK;
-    extern __shared__ __align__(16) double s_f[];
-    __shared__ PSum s_ps[FIELD_SCAN / 32 + 1];
-    __shared__ double s_Ew[2];
+    extern __shared__ __align__(16) unsigned long long s_f[];
+    __shared__ unsigned long long s_ps[6][FIELD_SUMS], s_tot[6];
+    __shared__ double s_g1;
+    __shared__ Current s_J;  // of one thread, kept out of its registers
     __shared__ int s_err;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    grid_dep_sync();
+    const int d = blockIdx.y >> 1, part = (int)blockIdx.x - nsl;
     if (tid == 0) s_err = 0;
     __syncthreads();
-    if ((int)blockIdx.x < nsl) {
+    grid_dep_sync();
+    if (part < 0) {
         seg_apply<BLOCK>(discs, ctl, out_buf, tid, lane, warp);
-    } else if ((mode & 1) && (blockIdx.y & 1) == 1) {  // store totals of discharge y / 2
-        if (warp == 0) {
-            int e2 = 0;
-            store_totals(discs[blockIdx.y >> 1], blockIdx.y >> 1, ctl, lane, ctl->slice_par, (mode & 2) != 0, out_buf,
-                         e2);
-            if (e2 && lane == 0) atomicOr(&s_err, e2);
-        }
-    } else if (!(mode & 8) && (blockIdx.y & 1) == 0) {
-        field_solve<T>(discs[blockIdx.y >> 1], blockIdx.y >> 1, ctl, mode, tid, lane, warp, s_f, max_N, s_ps, s_Ew);
+    } else if ((blockIdx.y & 1) == 0) {
+        if (!(mode & 8)) field_solve<T>(discs[d], d, ctl, mode, part, tid, lane, warp, s_f, max_N, s_ps, s_tot, &s_g1, s_J);
+    } else if (part > 0) {
+        if (!(mode & 8)) moments_part(discs[d], d, ctl, mode, part - 1, tid);
+    } else if ((mode & 1) && warp == 0) {  // store totals
+        int e2 = 0;
+        store_totals(discs[d], d, ctl, lane, ctl->slice_par, (mode & 2) != 0, out_buf, e2);
+        if (e2 && lane == 0) atomicOr(&s_err, e2);
     }
     __syncthreads();
-    // the last CTA advances the step (bit 2) and, after a sweep, the slice parity. Every CTA has
-    // consumed its reads of both before its count (data dependence), and the last CTA reads no other
-    // CTA's results, so no fence: the kernel boundary publishes everything
+    // the last CTA advances the step (bit 2) and the parities. Every CTA has consumed its reads of all
+    // three before its count (data dependence), and the last CTA reads no other CTA's results, so no
+    // fence: the kernel boundary publishes everything
     if (tid == 0) {
         if (s_err) atomicOr(&ctl->error, s_err);
         const unsigned prev = atomicAdd(&ctl->fin_done, 1u);
@@ -1462,6 +1555,7 @@ __global__ void __launch_bounds__(POST_BLOCK, 1) k_post(const Disc* __restrict__
             ctl->fin_done = 0;
             if (mode & 2) ctl->step = ctl->step + 1;
             if (mode & 1) ctl->slice_par = ctl->slice_par ^ 1;
+            if (!(mode & 8)) ctl->dep_par = ctl->dep_par ^ 1;
         }
     }
 }
@@ -1572,7 +1666,7 @@ __global__ void k_deposit(const Disc* __restrict__ discs, const Ctl* __restrict_
     }
     __syncthreads();
     for (int j = threadIdx.x; j <= N; j += blockDim.x)
-        if (s_h[j]) atomicAdd(&D.D[sp][j], s_h[j]);
+        if (s_h[j]) atomicAdd(&D.D[sp][(size_t)ctl->dep_par * (N + 1) + j], s_h[j]);
 }
 
 // Half back-kick after the initial solve: stored v_z = v_0 - (q/m) E_0 dt / 2.
@@ -2280,7 +2374,7 @@ static cudaError_t smem_attr(K kern, size_t smem) {
 // the kernel-to-kernel gap of a step shrinks while the ordering stays that of plain launches.
 template <typename... KArgs, typename... Args>
 static cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                              Args... args) {
+                             Args... args) {
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -2294,70 +2388,63 @@ static cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
-template <typename T, int BLOCK, int PPT>
+template <typename T, int PPT>
 static cudaError_t launch_sweep_t(const SweepLaunch& L) {
-    const size_t smem = sweep_smem<T, BLOCK, PPT>(L.max_N, L.n_disc);
-    auto kern = k_sweep<T, BLOCK, PPT>;
+    const size_t smem = sweep_smem<T, PPT>(L.max_N, L.sets, L.warps, L.n_disc);
+    auto kern = k_sweep<T, PPT>;
     cudaError_t e = smem_attr(kern, smem);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(kern, dim3(L.grid), dim3(BLOCK), smem, L.stream, L.discs, L.n_disc, L.ctl, L.in_buf, L.seed,
-                   L.max_N);
+    e = launch_pdl(kern, dim3(L.grid), dim3(32 * L.warps), smem, L.stream, L.discs, L.n_disc, L.ctl, L.in_buf, L.seed,
+                   L.max_N, L.sets);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
 template <typename T>
 static cudaError_t launch_sweep_p(const SweepLaunch& L) {
-    if (L.block == 512) {
-        if (L.ppt == 2) return launch_sweep_t<T, 512, 2>(L);
-        return launch_sweep_t<T, 512, 4>(L);
-    }
-    if (L.block == 128) {
-        if (L.ppt == 2) return launch_sweep_t<T, 128, 2>(L);
-        if (L.ppt == 8) return launch_sweep_t<T, 128, 8>(L);
-        return launch_sweep_t<T, 128, 4>(L);
-    }
-    if (L.ppt == 2) return launch_sweep_t<T, 256, 2>(L);
-    if (L.ppt == 8) return launch_sweep_t<T, 256, 8>(L);
-    return launch_sweep_t<T, 256, 4>(L);
+    if (L.ppt == 2) return launch_sweep_t<T, 2>(L);
+    if (L.ppt == 8) return launch_sweep_t<T, 8>(L);
+    return launch_sweep_t<T, 4>(L);
 }
 
 cudaError_t launch_sweep(const SweepLaunch& L) {
     return L.fp64 ? launch_sweep_p<double>(L) : launch_sweep_p<float>(L);
 }
 
-template <typename T, int BLOCK, int PPT>
-static int occ_t(int max_N, int n_disc) {
-    int nb = 0;
-    const size_t smem = sweep_smem<T, BLOCK, PPT>(max_N, n_disc);
-    smem_attr(k_sweep<T, BLOCK, PPT>, smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_sweep<T, BLOCK, PPT>, BLOCK, smem);
-    return nb;
+// Warps of a sweep CTA and its histogram sets. As many warps as registers and shared memory hold, but
+// no more than the CTA's share of the chunks (small stores: a smaller CTA starts faster) and at least 4;
+// two sets (no barrier between a discharge's electrons and ions) unless the second set costs more than
+// a quarter of the warps (above about 2900 cells).
+template <typename T, int PPT>
+static void sweep_shape_t(int max_N, int n_disc, int want, long long chunks, int* warps, int* sets) {
+    constexpr unsigned LIMIT = 227 * 1024 - 4096;  // the static part is below 4 KB
+    const int top = sweep_max_threads<T>() / 32;
+    int fit[3] = {0, 0, 0};
+    for (int s = 1; s <= 2; ++s)
+        for (int w = 1; w <= top && sweep_smem<T, PPT>(max_N, s, w, n_disc) <= LIMIT; ++w) fit[s] = w;
+    *sets = 4 * fit[2] >= 3 * fit[1] ? 2 : 1;
+    int w = fit[*sets];
+    if (want > 0 && want < w) w = want;
+    if (chunks < w) w = (int)chunks;
+    *warps = w < 4 ? (fit[*sets] < 4 ? fit[*sets] : 4) : w;  // at least 2 fit at any size
 }
-template <typename T>
-static int occ_p(int block, int ppt, int max_N, int n_disc) {
-    if (block == 512) {
-        if (ppt == 2) return occ_t<T, 512, 2>(max_N, n_disc);
-        return occ_t<T, 512, 4>(max_N, n_disc);
+void sweep_shape(int fp64, int ppt, int max_N, int n_disc, int want, long long chunks, int* warps, int* sets) {
+    if (fp64) {
+        if (ppt == 2) return sweep_shape_t<double, 2>(max_N, n_disc, want, chunks, warps, sets);
+        if (ppt == 8) return sweep_shape_t<double, 8>(max_N, n_disc, want, chunks, warps, sets);
+        return sweep_shape_t<double, 4>(max_N, n_disc, want, chunks, warps, sets);
     }
-    if (block == 128) {
-        if (ppt == 2) return occ_t<T, 128, 2>(max_N, n_disc);
-        if (ppt == 8) return occ_t<T, 128, 8>(max_N, n_disc);
-        return occ_t<T, 128, 4>(max_N, n_disc);
-    }
-    if (ppt == 2) return occ_t<T, 256, 2>(max_N, n_disc);
-    if (ppt == 8) return occ_t<T, 256, 8>(max_N, n_disc);
-    return occ_t<T, 256, 4>(max_N, n_disc);
-}
-int sweep_occupancy(int fp64, int block, int ppt, int max_N, int n_disc) {
-    return fp64 ? occ_p<double>(block, ppt, max_N, n_disc) : occ_p<float>(block, ppt, max_N, n_disc);
+    if (ppt == 2) return sweep_shape_t<float, 2>(max_N, n_disc, want, chunks, warps, sets);
+    if (ppt == 8) return sweep_shape_t<float, 8>(max_N, n_disc, want, chunks, warps, sets);
+    sweep_shape_t<float, 4>(max_N, n_disc, want, chunks, warps, sets);
 }
 
 cudaError_t launch_finalize(int fp64, const Disc* discs, int n_disc, Ctl* ctl, int out_buf, int mode, int max_slices,
                             int max_N, cudaStream_t st) {
-    const size_t smem = sizeof(double) * 2 * ((size_t)max_N + 1);
+    const size_t smem = (mode & 8) ? 0 : sizeof(unsigned long long) * 2 * ((size_t)max_N + 1);
     const int nsl = (mode & 1) ? (max_slices > 0 ? max_slices : 1) : 0;
-    const dim3 grid(nsl + 1, 2 * n_disc);
+    const int parts = (mode & 8) ? 1 : max_N / FIELD_NODES + 2;  // field parts (y even), totals and moments parts (odd)
+    const dim3 grid(nsl + parts, 2 * n_disc);
     if (fp64) {
         smem_attr(k_post<double>, smem);
         return launch_pdl(k_post<double>, grid, dim3(POST_BLOCK), smem, st, discs, n_disc, ctl, out_buf, mode, nsl,

@@ -5,7 +5,8 @@
 namespace pic {
 
 struct SweepLaunch {
-    int fp64, block, ppt, grid, max_N, n_disc, in_buf;
+    int fp64, ppt, grid, max_N, n_disc, in_buf;
+    int warps, sets;  // of sweep_shape
     const Disc* discs;
     Ctl* ctl;
     unsigned long long seed;
@@ -13,7 +14,9 @@ struct SweepLaunch {
 };
 
 cudaError_t launch_sweep(const SweepLaunch& L);
-int sweep_occupancy(int fp64, int block, int ppt, int max_N, int n_disc);
+// Shape of the sweep's CTAs (one per SM): warps and histogram sets, see sweep_shape in pic_kernels.cu.
+// want: the caller's limit on warps (0: none); chunks: of all stores at capacity, per SM.
+void sweep_shape(int fp64, int ppt, int max_N, int n_disc, int want, long long chunks, int* warps, int* sets);
 cudaError_t launch_finalize(int fp64, const Disc* discs, int n_disc, Ctl* ctl, int out_buf, int mode, int max_slices,
                             int max_N, cudaStream_t st);
 cudaError_t launch_load(int fp64, const Disc* discs, int n_disc, Ctl* ctl, int buf, unsigned long long seed,
