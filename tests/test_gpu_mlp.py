@@ -118,3 +118,29 @@ def test_rejects_batches_beyond_capacity(N):
     with pytest.raises(RuntimeError):
         net.forward(np.zeros((9, RAGGED[0]), np.float32))
     net.close()
+
+
+# Products at the edges of their tiles (128 rows, 16 / 32 / 64 columns, K chunks of 128, a ring of four) and
+# a batch smaller than the one before (its padding must not keep the larger batch's rows).
+EDGES = [([16, 16, 16], 16), ([17, 31, 33], 129), ([129, 128, 127], 128), ([130, 513, 15], 131),
+         ([300, 1100, 48], 260), ([3, 2, 1], 2), ([5, 640, 640, 7], 1)]
+
+
+@pytest.mark.parametrize("sizes,batch", EDGES)
+def test_tile_edges_match_oracle(N, sizes, batch):
+    rng = np.random.default_rng(sum(sizes) + batch)
+    net = N.MLP(sizes, max_batch=batch + 40, seed=3)
+    p = M.weights_bf16(net.get_params(), sizes)
+    for b in (batch + 40, batch):
+        x = rng.standard_normal((b, sizes[0])).astype(np.float32)
+        t = rng.standard_normal((b, sizes[-1])).astype(np.float32)
+        y = net.forward(x).cpu().numpy()
+        assert _rel(y, M.forward(p, sizes, x)[-1]) < 2e-2
+        loss = net.loss_grad(x, t)
+        ref_loss, ref_g = M.loss_grad(p, sizes, x, t)
+        assert abs(loss - ref_loss) <= 1e-2 * ref_loss
+        g = net.grads()
+        for (w, o, i, n) in M.layout(sizes)[0]:
+            assert _rel(g[w:w + i * n], ref_g[w:w + i * n]) < 3e-2
+            assert _rel(g[o:o + n], ref_g[o:o + n]) < 3e-2
+    net.close()
