@@ -46,8 +46,9 @@ struct pic_ctx {
     unsigned* sort_hist = nullptr;
     unsigned* sort_tot = nullptr;
     long long* sort_hoff = nullptr;
-    unsigned* sort_kr = nullptr;    // per slot of every store: cell | rank in its sort tile << 16
-    long long* sort_eoff = nullptr; // first slot of each store in sort_kr
+    unsigned* sort_kr = nullptr;    // per slot of every store's sort tiles: cell | rank in its tile << 16
+    long long* sort_eoff = nullptr; // first entry of each store in sort_kr
+    long long max_tiles = 0;        // sort tiles of all stores at most
     int repack_every = 0;           // order-preserving repack after every step n with (n+1) % this == 0
     std::vector<void*> allocs;
     int cur = 0;
@@ -421,7 +422,12 @@ extern "C" pic_status pic_batch_create(pic_ctx** out, const pic_gas* gases, int3
         for (int i = 0; i < n_dis; ++i)
             for (int sp = 0; sp < 2; ++sp) {
                 eoff[2 * i + sp] = ea;
-                ea += sp ? ctx->dis[i].weights.capacity_i : ctx->dis[i].weights.capacity_e;
+                const long long cap = sp ? ctx->dis[i].weights.capacity_i : ctx->dis[i].weights.capacity_e;
+                // by tile, so with room for the gaps of a region layout
+                const long long st = sort_tile_chunks((int)chunk);
+                const long long tiles = (region_sizes(cap, chunk, bcap_of(i)).maxchunks + st - 1) / st;
+                ctx->max_tiles += tiles;
+                ea += tiles * st * chunk;
             }
         ALLOC(ctx->sort_kr, unsigned*, sizeof(unsigned) * (size_t)std::max(ea, 1ll));
         ALLOC(ctx->sort_eoff, long long*, sizeof(long long) * 2 * MAXD);
@@ -715,10 +721,9 @@ static pic_status enqueue_finalize(pic_ctx* ctx, int mode) {
 }
 
 static pic_status enqueue_sort(pic_ctx* ctx) {
-    const int gx = std::max(1, ctx->num_sms * 2);
     CK(launch_sort(ctx->fp64, ctx->d_discs, ctx->n_disc, ctx->d_ctl, ctx->cur, 1 - ctx->cur, ctx->sort_hist,
-                   ctx->sort_hoff, ctx->sort_tot, ctx->sort_kr, ctx->sort_eoff, ctx->max_N, gx,
-                   ctx->stream),
+                   ctx->sort_hoff, ctx->sort_tot, ctx->sort_kr, ctx->sort_eoff, ctx->max_N, ctx->max_tiles,
+                   std::max(1, ctx->num_sms), ctx->stream),
        "sort launch");
     ctx->cur = 1 - ctx->cur;
     return PIC_OK;

@@ -1914,97 +1914,155 @@ __global__ void __launch_bounds__(DIAG_BLOCK) k_diag(const Disc* __restrict__ di
         if (s_eedf[j]) atomicAdd(&D.dg_eedf[j], (unsigned long long)s_eedf[j]);
 }
 
-// Stable counting sort by cell. A sort tile is SORT_NW warps of SORT_R rows of 32 slots: warp w of
-// tile t walks the store's chunks t SORT_NW CPW + w CPW .. + CPW - 1 (CPW = SORT_R 32 / CHUNK) in
-// slot order.
-constexpr int SORT_BLOCK = 256, SORT_NW = SORT_BLOCK / 32, SORT_R = 16;
+// Stable counting sort of every store by cell into the other buffer (dense):
+//   k_sort_count   tiles of 4096 slots: each slot's cell and its rank among the tile's slots of the same
+//                  cell (in slot order), packed into kr, and the tile's cell counts into hist[t N + c];
+//   k_sort_rows    per cell: exclusive scan of the counts over the tiles; the last CTA of a store scans the
+//                  cell totals (first slot of every cell);
+//   k_sort_scatter the same tiles: destination = first slot of its cell + the tile's offset in that cell +
+//                  its rank.
+// The first and last run over one list of the tiles of all stores: with a CTA per (store, possible tile), 64
+// discharges of 2e4 + 2e4 launched 38912 CTAs, most of them empty, in 72 us each. A tile: warp w walks chunks
+// t SORT_NW CPW + w CPW .. + CPW - 1 (CPW = SORT_R 32 / CHUNK) in slot order. What bounds them is latency (of
+// the loads, and of the warp's serial ranks), so many warps with the loads of several rows in flight: 16-bit
+// counters, offsets of 4 rows at a time. Measured on aged stores, the three kernels: 31.5
+// -> 25 us at 2e4 + 2e4 particles (128 cells), 157 -> 67 for 64 such discharges, 40 -> 37 at 1e6 + 1e6
+// (512), 466 -> 366 at 1.2e7 + 1.2e7 (2048). Sorting a store of 2.5e4 whole by one CTA took 40 us.
+constexpr int SORT_BLOCK = 512, SORT_NW = SORT_BLOCK / 32, SORT_R = 8, SORT_TILE = SORT_BLOCK * SORT_R;
 __device__ __forceinline__ long long sort_tiles(long long chunks, int chunk) {
     const long long per = (long long)SORT_NW * (SORT_R * 32 / chunk);
     return (chunks + per - 1) / per;
 }
+// The list: per store the tiles before it. Called by all threads; s_pre has 2 n_disc + 1 entries.
+__device__ __forceinline__ void sort_list(const Disc* __restrict__ discs, const Ctl* ctl, int n_disc, int buf, int* s_pre) {
+    const int n_store = 2 * n_disc;
+    for (int s = threadIdx.x; s < n_store; s += blockDim.x) {
+        const int d = s >> 1, sp = s & 1;
+        s_pre[s + 1] = (int)sort_tiles(chunks_of(ctl->lay[d][sp][buf], ctl->count[d][sp], discs[d].chunk), discs[d].chunk);
+    }
+    if (threadIdx.x == 0) s_pre[0] = 0;
+    __syncthreads();
+    if (threadIdx.x < 32) {  // inclusive prefix over at most 128 stores, four per lane
+        const int lane = threadIdx.x, b = 4 * lane + 1;
+        int v[4], x = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            v[i] = b + i <= n_store ? s_pre[b + i] : 0;
+            x += v[i];
+        }
+        int y = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int z = __shfl_up_sync(FULL, y, o);
+            if (lane >= o) y += z;
+        }
+        y -= x;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            y += v[i];
+            if (b + i <= n_store) s_pre[b + i] = y;
+        }
+    }
+    __syncthreads();
+}
+__device__ __forceinline__ int sort_store(const int* s_pre, int n_store, int item) {  // last store with s_pre <= item
+    int lo = 0, hi = n_store - 1;
+    while (lo < hi) {
+        const int m = (lo + hi + 1) >> 1;
+        if (s_pre[m] <= item) lo = m;
+        else hi = m - 1;
+    }
+    return lo;
+}
 
-// Stable counting sort of every store by cell:
-//   k_sort_count   per tile: each slot's cell and its rank among the tile's
-//                  slots of the same cell (in slot order), packed with the cell
-//                  into kr[slot], and the tile's cell counts into
-//                  hist[seg][t N + c];
-//   k_sort_rows    per cell: exclusive scan of the counts over the tiles; the
-//                  last CTA of a store scans the cell totals (first slot of
-//                  every cell);
-//   k_sort_scatter per tile, walking the same chunks: destination = first slot
-//                  of its cell + the tile's offset in that cell + its rank; the
-//                  sorted buffer's layout is dense.
-__global__ void __launch_bounds__(SORT_BLOCK) k_sort_count(const Disc* __restrict__ discs, const Ctl* __restrict__ ctl,
-                                                           int buf, unsigned* __restrict__ hist,
+// Ranks of a row of 32 slots among the equal cells of its warp so far, and the warp's counters (16 bits per
+// cell) advanced. k >= N: not placed. Returns the rank.
+__device__ __forceinline__ unsigned row_rank(unsigned short* W, unsigned k, unsigned N, int lane, unsigned lt) {
+    const unsigned k0 = __shfl_sync(FULL, k, 0);
+    unsigned rank = 0;
+    if (__all_sync(FULL, k == k0)) {  // the rule on a nearly sorted store of slow particles
+        if (k0 < N) {
+            rank = W[k0] + lane;
+            __syncwarp();
+            if (lane == 31) W[k0] = (unsigned short)(rank + 1);
+        }
+    } else {
+        const unsigned peers = __match_any_sync(FULL, k);
+        if (k < N) {
+            const unsigned b = W[k];
+            rank = b + __popc(peers & lt);
+            __syncwarp(peers);
+            if (lane == __ffs(peers) - 1) W[k] = (unsigned short)(b + __popc(peers));
+        }
+    }
+    __syncwarp();
+    return rank;
+}
+
+__global__ void __launch_bounds__(SORT_BLOCK, 3) k_sort_count(const Disc* __restrict__ discs, int n_disc,
+                                                           Ctl* __restrict__ ctl, int src, int dst,
+                                                           unsigned* __restrict__ hist,
                                                            const long long* __restrict__ hoff,
                                                            unsigned* __restrict__ kr_all,
                                                            const long long* __restrict__ eoff, int max_N) {
-    grid_dep_sync();
-    extern __shared__ __align__(16) unsigned s_w[];  // [SORT_NW][max_N] per-warp counts, then prefixes
-    const int seg = blockIdx.y, d = seg >> 1, sp = seg & 1;
-    const Disc& D = discs[d];
-    const int N = D.N, CHUNK = D.chunk, RPC = CHUNK / 32, CPW = SORT_R / RPC;
-    const long long n = ctl->count[d][sp];
-    const Lay L = ctl->lay[d][sp][buf];
-    const long long chunks = chunks_of(L, n, CHUNK);
-    const long long Ts = sort_tiles(chunks, CHUNK);
-    const int32_t* __restrict__ cc = D.c[buf][sp];
-    const int* st = D.start[sp];
-    unsigned* H = hist + hoff[seg];
-    unsigned* KR = kr_all + eoff[seg];
+    extern __shared__ __align__(16) unsigned short s_w[];  // [SORT_NW][nw2] counts, then prefixes
+    __shared__ int s_pre[2 * MAXD + 1];
+    const int nw2 = (max_N + 1) / 2 * 2;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    unsigned* Wc = s_w + warp * max_N;
-    for (long long t = blockIdx.x; t < Ts; t += gridDim.x) {
-        for (int j = tid; j < SORT_NW * max_N; j += SORT_BLOCK) s_w[j] = 0;
-        __syncthreads();
-        const long long k0 = (t * SORT_NW + warp) * CPW;
+    unsigned short* W = s_w + warp * nw2;
+    grid_dep_sync();
+    sort_list(discs, ctl, n_disc, src, s_pre);
+    if (blockIdx.x == 0)  // every sorted store is dense
+        for (int s = tid; s < 2 * n_disc; s += SORT_BLOCK) ctl->lay[s >> 1][s & 1][dst] = Lay{0, 0, 0, 0};
+    const int items = s_pre[2 * n_disc];
+    for (int item = blockIdx.x; item < items; item += gridDim.x) {
+        const int seg = sort_store(s_pre, 2 * n_disc, item), d = seg >> 1, sp = seg & 1;
+        const Disc& D = discs[d];
+        const long long n = ctl->count[d][sp];
+        const Lay L = ctl->lay[d][sp][src];
+        const int N = D.N, CHUNK = D.chunk, rs = __ffs(CHUNK) - 6, rm = (1 << rs) - 1, CPW = SORT_R >> rs;
+        const int t = item - s_pre[seg];
+        const long long chunks = chunks_of(L, n, CHUNK);
+        const int32_t* __restrict__ cc = D.c[src][sp];
+        for (int j = tid; j < SORT_NW * nw2 / 2; j += SORT_BLOCK) reinterpret_cast<unsigned*>(s_w)[j] = 0;
+        const long long k0 = ((long long)t * SORT_NW + warp) * CPW;
+        // the warp's chunk descriptors by its first lanes, then all cell loads
+        const ChunkDesc my = lane < CPW && k0 + lane < chunks ? chunk_desc(L, n, D.start[sp], k0 + lane, CHUNK)
+                                                             : ChunkDesc{0, 0, 0};
         unsigned kr[SORT_R];
-        int slot[SORT_R];
-        ChunkDesc cd{0, 0, 0};
 #pragma unroll
-        for (int r = 0; r < SORT_R; ++r) {  // all cell loads first
-            const int ci = r / RPC, row = r % RPC;
-            if (row == 0) cd = (k0 + ci < chunks) ? chunk_desc(L, n, st, k0 + ci, CHUNK) : ChunkDesc{0, 0, 0};
-            const int i = 32 * row + lane;
-            kr[r] = 0xFFFFu;
-            slot[r] = -1;
-            if (i < cd.cnt) {
-                kr[r] = (unsigned)__ldcs(cc + cd.src + i);  // checked below, after all loads are issued
-                slot[r] = cd.base + i;
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < SORT_R; ++r) {  // rank among the warp's equal cells so far
-            if (kr[r] >= (unsigned)N) kr[r] = 0xFFFFu;  // past the store, or a corrupt cell index: not placed
-            const int k = (int)kr[r];
-            const unsigned peers = __match_any_sync(FULL, k);
-            if (k < N) {
-                const unsigned b = Wc[k];
-                kr[r] |= (b + __popc(peers & lt)) << 16;
-                __syncwarp(peers);
-                if (lane == __ffs(peers) - 1) Wc[k] = b + __popc(peers);
-            }
-            __syncwarp();
-        }
-        __syncthreads();
-        for (int j = tid; j < N; j += SORT_BLOCK) {  // per cell: prefix over the warps, tile count
-            unsigned run = 0;
-#pragma unroll
-            for (int w = 0; w < SORT_NW; ++w) {
-                const unsigned v = s_w[w * max_N + j];
-                s_w[w * max_N + j] = run;
-                run += v;
-            }
-            H[(size_t)t * N + j] = run;
+        for (int r = 0; r < SORT_R; ++r) {
+            const int ci = r >> rs, i = 32 * (r & rm) + lane;
+            const int s0 = __shfl_sync(FULL, (int)my.src, ci), cnt = __shfl_sync(FULL, my.cnt, ci);
+            kr[r] = i < cnt ? (unsigned)__ldcs(cc + s0 + i) : 0xFFFFu;
         }
         __syncthreads();
 #pragma unroll
         for (int r = 0; r < SORT_R; ++r) {
-            if (slot[r] >= 0) {
-                const int k = (int)(kr[r] & 0xFFFFu);
-                KR[slot[r]] = k < N ? (unsigned)k | ((Wc[k] + (kr[r] >> 16)) << 16) : 0xFFFFu;
+            if (kr[r] >= (unsigned)N) kr[r] = 0xFFFFu;  // past the store, or a corrupt cell index: not placed
+            kr[r] |= row_rank(W, kr[r], N, lane, lt) << 16;
+        }
+        __syncthreads();
+        unsigned* H = hist + hoff[seg] + (size_t)t * N;
+        for (int j = tid; j < (N + 1) / 2; j += SORT_BLOCK) {  // two cells per word: prefix over the warps, tile counts
+            unsigned run = 0;
+#pragma unroll
+            for (int w = 0; w < SORT_NW; ++w) {
+                unsigned* p = reinterpret_cast<unsigned*>(s_w + w * nw2) + j;
+                const unsigned v = *p;
+                *p = run;
+                run += v;
             }
+            H[2 * j] = run & 0xFFFFu;
+            if (2 * j + 1 < N) H[2 * j + 1] = run >> 16;
+        }
+        __syncthreads();
+        unsigned* KR = kr_all + eoff[seg] + (size_t)t * SORT_TILE + warp * (32 * SORT_R) + lane;
+#pragma unroll
+        for (int r = 0; r < SORT_R; ++r) {
+            const unsigned k = kr[r] & 0xFFFFu;
+            KR[32 * r] = k < (unsigned)N ? kr[r] + ((unsigned)W[k] << 16) : 0xFFFFu;
         }
         __syncthreads();
     }
@@ -2065,18 +2123,25 @@ __global__ void __launch_bounds__(1024) k_sort_rows(const Disc* __restrict__ dis
     unsigned* H = hist + hoff[seg];
     const unsigned per = (Ts + 31) / 32, t0 = min(Ts, warp * per), t1 = min(Ts, t0 + per);
     unsigned sum = 0;
-    if (c < N)
+    if (c < N) {
+#pragma unroll 8
         for (unsigned t = t0; t < t1; ++t) sum += H[(size_t)t * N + c];
+    }
     s_sum[warp][lane] = sum;
     __syncthreads();
     unsigned pre = 0;
     for (int w = 0; w < warp; ++w) pre += s_sum[w][lane];
     if (warp == 31 && c < N) tot[(long long)seg * MAXN + c] = pre + sum;
     if (c < N)
-        for (unsigned t = t0; t < t1; ++t) {
-            const unsigned v = H[(size_t)t * N + c];
-            H[(size_t)t * N + c] = pre;
-            pre += v;
+        for (unsigned t = t0; t < t1; t += 8) {  // eight loads in flight
+            unsigned v[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = t + q < t1 ? H[(size_t)(t + q) * N + c] : 0u;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                if (t + q < t1) H[(size_t)(t + q) * N + c] = pre;
+                pre += v[q];
+            }
         }
     // the last CTA of the store turns the row totals into the first slot of every cell
     __shared__ int s_last;
@@ -2094,47 +2159,60 @@ __global__ void __launch_bounds__(1024) k_sort_rows(const Disc* __restrict__ dis
 }
 
 template <typename T>
-__global__ void __launch_bounds__(SORT_BLOCK) k_sort_scatter(const Disc* __restrict__ discs,
-                                                             Ctl* __restrict__ ctl, int src, int dst,
+__global__ void __launch_bounds__(SORT_BLOCK) k_sort_scatter(const Disc* __restrict__ discs, int n_disc,
+                                                             const Ctl* __restrict__ ctl, int src, int dst,
                                                              const unsigned* __restrict__ hist,
                                                              const long long* __restrict__ hoff,
                                                              const unsigned* __restrict__ tot,
                                                              const unsigned* __restrict__ kr_all,
                                                              const long long* __restrict__ eoff) {
+    __shared__ int s_pre[2 * MAXD + 1];
     grid_dep_sync();
-    const int seg = blockIdx.y, d = seg >> 1, sp = seg & 1;
-    const Disc& D = discs[d];
-    const int N = D.N, CHUNK = D.chunk, RPC = CHUNK / 32, CPW = SORT_R / RPC;
-    const long long n = ctl->count[d][sp];
-    const Lay L = ctl->lay[d][sp][src];
-    const long long chunks = chunks_of(L, n, CHUNK);
-    const long long Ts = sort_tiles(chunks, CHUNK);
+    sort_list(discs, ctl, n_disc, src, s_pre);
     using R = typename Rec<T>::type;
-    const R* __restrict__ ps = reinterpret_cast<const R*>(D.p[src][sp]);
-    R* __restrict__ pd = reinterpret_cast<R*>(D.p[dst][sp]);
-    int32_t* __restrict__ cd = D.c[dst][sp];
-    const int* st = D.start[sp];
-    const unsigned* H = hist + hoff[seg];
-    const unsigned* cstart = tot + (long long)seg * MAXN;
-    const unsigned* KR = kr_all + eoff[seg];
+    constexpr int B = sizeof(T) == 4 ? 4 : 2;  // rows whose loads go out together
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->lay[d][sp][dst] = Lay{0, 0, 0, 0};  // the sorted store is dense
-    for (long long t = blockIdx.x; t < Ts; t += gridDim.x) {
-        const long long k0 = (t * SORT_NW + warp) * CPW;
-        for (int ci = 0; ci < CPW && k0 + ci < chunks; ++ci) {
-            const ChunkDesc c = chunk_desc(L, n, st, k0 + ci, CHUNK);
-            for (int row = 0; row < RPC; ++row) {
-                const int i = 32 * row + lane;
-                if (i >= c.cnt) continue;
-                const unsigned kr = __ldcs(KR + c.base + i);
-                const int k = (int)(kr & 0xFFFFu);
-                if (k >= N) continue;  // a corrupt cell index (reported by the sweep): dropped
-                const unsigned long long o = (unsigned long long)cstart[k] + H[(size_t)t * N + k] + (kr >> 16);
-                if (o < (unsigned long long)n) {
-                    cd[o] = k;
-                    pd[o] = ps[c.src + i];
-                }
+    const int items = s_pre[2 * n_disc];
+    for (int item = blockIdx.x; item < items; item += gridDim.x) {
+        const int seg = sort_store(s_pre, 2 * n_disc, item), d = seg >> 1, sp = seg & 1;
+        const Disc& D = discs[d];
+        const int N = D.N, CHUNK = D.chunk, rs = __ffs(CHUNK) - 6, rm = (1 << rs) - 1, CPW = SORT_R >> rs;
+        const int t = item - s_pre[seg];
+        const long long n = ctl->count[d][sp];
+        const Lay L = ctl->lay[d][sp][src];
+        const long long chunks = chunks_of(L, n, CHUNK), k0 = ((long long)t * SORT_NW + warp) * CPW;
+        const R* __restrict__ ps = reinterpret_cast<const R*>(D.p[src][sp]);
+        R* __restrict__ pd = reinterpret_cast<R*>(D.p[dst][sp]);
+        int32_t* __restrict__ cd = D.c[dst][sp];
+        const unsigned* __restrict__ H = hist + hoff[seg] + (size_t)t * N;
+        const unsigned* __restrict__ cstart = tot + (long long)seg * MAXN;
+        const unsigned* __restrict__ KR = kr_all + eoff[seg] + (size_t)t * SORT_TILE + warp * (32 * SORT_R) + lane;
+        const ChunkDesc my = lane < CPW && k0 + lane < chunks ? chunk_desc(L, n, D.start[sp], k0 + lane, CHUNK)
+                                                             : ChunkDesc{0, 0, 0};
+#pragma unroll 1
+        for (int r0 = 0; r0 < SORT_R; r0 += B) {
+            unsigned kr[B], o[B];
+            R rec[B];
+#pragma unroll
+            for (int q = 0; q < B; ++q) kr[q] = __ldcs(KR + 32 * (r0 + q));
+#pragma unroll
+            for (int q = 0; q < B; ++q) {
+                const int r = r0 + q, i = 32 * (r & rm) + lane;
+                const int s0 = __shfl_sync(FULL, (int)my.src, r >> rs), cnt = __shfl_sync(FULL, my.cnt, r >> rs);
+                if (i < cnt) rec[q] = ps[s0 + i];
+                else kr[q] = 0xFFFFu;
             }
+#pragma unroll
+            for (int q = 0; q < B; ++q) {
+                const unsigned k = kr[q] & 0xFFFFu;  // a corrupt cell index (reported by the sweep): dropped
+                o[q] = k < (unsigned)N ? cstart[k] + H[k] + (kr[q] >> 16) : 0xFFFFFFFFu;
+            }
+#pragma unroll
+            for (int q = 0; q < B; ++q)
+                if (o[q] < (unsigned long long)n) {
+                    cd[o[q]] = (int)(kr[q] & 0xFFFFu);
+                    pd[o[q]] = rec[q];
+                }
         }
     }
 }
@@ -2524,12 +2602,15 @@ cudaError_t launch_tables(int fp64, int n_pts, int n_proc, double de, double M, 
 
 cudaError_t launch_sort(int fp64, const Disc* discs, int n_disc, Ctl* ctl, int src, int dst, unsigned* hist,
                         const long long* hoff, unsigned* tot, unsigned* kr, const long long* eoff, int max_N,
-                        int grid_x, cudaStream_t st) {
-    dim3 g(grid_x, 2 * n_disc);
-    const size_t smem = sizeof(unsigned) * SORT_NW * max_N;
+                        long long max_tiles, int sms, cudaStream_t st) {
+    // CTAs: what the SMs hold (the counters take 32 bytes a cell), but not more than there can be tiles
+    const size_t smem = 2 * (size_t)SORT_NW * ((max_N + 1) / 2 * 2);
+    const int per = smem > 100 * 1024 ? 1 : smem > 70 * 1024 ? 2 : 3;
+    auto grid = [&](int p) { return dim3((unsigned)(max_tiles < (long long)p * sms ? max_tiles : (long long)p * sms)); };
     cudaError_t e = smem_attr(k_sort_count, smem);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(k_sort_count, g, dim3(SORT_BLOCK), smem, st, discs, ctl, src, hist, hoff, kr, eoff, max_N);
+    e = launch_pdl(k_sort_count, grid(per), dim3(SORT_BLOCK), smem, st, discs, n_disc, ctl, src, dst, hist, hoff, kr, eoff,
+                   max_N);
     if (e != cudaSuccess) return e;
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -2539,10 +2620,10 @@ cudaError_t launch_sort(int fp64, const Disc* discs, int n_disc, Ctl* ctl, int s
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (fp64)
-        return launch_pdl(k_sort_scatter<double>, g, dim3(SORT_BLOCK), 0, st, discs, ctl, src, dst, hist, hoff, tot, kr,
-                          eoff);
-    return launch_pdl(k_sort_scatter<float>, g, dim3(SORT_BLOCK), 0, st, discs, ctl, src, dst, hist, hoff, tot, kr,
-                      eoff);
+        return launch_pdl(k_sort_scatter<double>, grid(3), dim3(SORT_BLOCK), 0, st, discs, n_disc, ctl, src, dst, hist, hoff,
+                          tot, kr, eoff);
+    return launch_pdl(k_sort_scatter<float>, grid(3), dim3(SORT_BLOCK), 0, st, discs, n_disc, ctl, src, dst, hist, hoff, tot,
+                      kr, eoff);
 }
 
 cudaError_t launch_repack(int fp64, const Disc* discs, int n_disc, Ctl* ctl, int src, int dst, int grid_x,
@@ -2575,7 +2656,7 @@ cudaError_t launch_unpack_state(int fp64, const Disc* discs, const Ctl* ctl, int
 }
 
 
-long long sort_tile_chunks(int chunk) { return (long long)SORT_NW * (SORT_R * 32 / chunk); }
+long long sort_tile_chunks(int chunk) { return SORT_TILE / chunk; }
 
 cudaError_t launch_finish_upload(const Disc* discs, Ctl* ctl, int d, int sp, long long n, const unsigned* bad,
                                  int buf, cudaStream_t st) {

@@ -29,7 +29,7 @@ cudaError_t launch_tables(int fp64, int n_pts, int n_proc, double de, double M, 
                           void* Te, void* Ti, unsigned long long* kmax, cudaStream_t st);
 cudaError_t launch_sort(int fp64, const Disc* discs, int n_disc, Ctl* ctl, int src, int dst, unsigned* hist,
                         const long long* hoff, unsigned* tot, unsigned* kr, const long long* eoff, int max_N,
-                        int grid_x, cudaStream_t st);
+                        long long max_tiles, int sms, cudaStream_t st);
 cudaError_t launch_repack(int fp64, const Disc* discs, int n_disc, Ctl* ctl, int src, int dst, int grid_x,
                           cudaStream_t st);
 // state transfer: cells and the four SoA value arrays (f, vx, vy, vz), in device staging or mapped
