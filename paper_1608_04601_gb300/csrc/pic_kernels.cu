@@ -22,6 +22,7 @@
 //               the electrons' node moments and energy histogram.
 #include "pic_internal.h"
 #include "pic_device.cuh"
+#include "pic_sort.cuh"
 
 namespace pic {
 
@@ -30,8 +31,6 @@ namespace pic {
 #define EPS0 8.8541878128e-12
 #define PI_D 3.14159265358979323846
 #define TWO32_D 4294967296.0
-
-constexpr unsigned FULL = 0xFFFFFFFFu;
 
 template <typename T> __device__ __forceinline__ const Consts<T>& consts_of(const Disc& d);
 template <> __device__ __forceinline__ const Consts<float>& consts_of<float>(const Disc& d) { return d.cf; }
@@ -1928,7 +1927,6 @@ __global__ void __launch_bounds__(DIAG_BLOCK) k_diag(const Disc* __restrict__ di
 // counters, offsets of 4 rows at a time. Measured on aged stores, the three kernels: 31.5
 // -> 25 us at 2e4 + 2e4 particles (128 cells), 157 -> 67 for 64 such discharges, 40 -> 37 at 1e6 + 1e6
 // (512), 466 -> 366 at 1.2e7 + 1.2e7 (2048). Sorting a store of 2.5e4 whole by one CTA took 40 us.
-constexpr int SORT_BLOCK = 512, SORT_NW = SORT_BLOCK / 32, SORT_R = 8, SORT_TILE = SORT_BLOCK * SORT_R;
 __device__ __forceinline__ long long sort_tiles(long long chunks, int chunk) {
     const long long per = (long long)SORT_NW * (SORT_R * 32 / chunk);
     return (chunks + per - 1) / per;
@@ -1973,30 +1971,6 @@ __device__ __forceinline__ int sort_store(const int* s_pre, int n_store, int ite
         else hi = m - 1;
     }
     return lo;
-}
-
-// Ranks of a row of 32 slots among the equal cells of its warp so far, and the warp's counters (16 bits per
-// cell) advanced. k >= N: not placed. Returns the rank.
-__device__ __forceinline__ unsigned row_rank(unsigned short* W, unsigned k, unsigned N, int lane, unsigned lt) {
-    const unsigned k0 = __shfl_sync(FULL, k, 0);
-    unsigned rank = 0;
-    if (__all_sync(FULL, k == k0)) {  // the rule on a nearly sorted store of slow particles
-        if (k0 < N) {
-            rank = W[k0] + lane;
-            __syncwarp();
-            if (lane == 31) W[k0] = (unsigned short)(rank + 1);
-        }
-    } else {
-        const unsigned peers = __match_any_sync(FULL, k);
-        if (k < N) {
-            const unsigned b = W[k];
-            rank = b + __popc(peers & lt);
-            __syncwarp(peers);
-            if (lane == __ffs(peers) - 1) W[k] = (unsigned short)(b + __popc(peers));
-        }
-    }
-    __syncwarp();
-    return rank;
 }
 
 __global__ void __launch_bounds__(SORT_BLOCK, 3) k_sort_count(const Disc* __restrict__ discs, int n_disc,
@@ -2068,94 +2042,17 @@ __global__ void __launch_bounds__(SORT_BLOCK, 3) k_sort_count(const Disc* __rest
     }
 }
 
-// Exclusive scan of one store's N row totals in place -> the first slot of every cell (1024
-// threads; the totals were written by other CTAs of the same grid, so they are read from L2).
-__device__ __forceinline__ void cells_scan(unsigned* a, int N) {
-    __shared__ unsigned s_v[MAXN];
-    __shared__ unsigned s_w[32];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int j = tid; j < N; j += 1024) s_v[j] = __ldcg(a + j);
-    __syncthreads();
-    const int per = (N + 1023) / 1024, lo = tid * per, hi = min(N, lo + per);
-    unsigned run = 0;
-    for (int j = lo; j < hi; ++j) run += s_v[j];
-    unsigned x = run;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned t = __shfl_up_sync(FULL, x, o);
-        if (lane >= o) x += t;
-    }
-    if (lane == 31) s_w[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-        const unsigned w = s_w[lane];
-        unsigned y = w;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned t = __shfl_up_sync(FULL, y, o);
-            if (lane >= o) y += t;
-        }
-        s_w[lane] = y - w;
-    }
-    __syncthreads();
-    unsigned e = s_w[warp] + x - run;
-    for (int j = lo; j < hi; ++j) {
-        const unsigned v = s_v[j];
-        a[j] = e;
-        e += v;
-    }
-}
-
-// Per (store, group of 32 cells): exclusive scan over the tiles in place (lane = cell, each warp
-// a contiguous range of tiles, so rows are read 128 bytes at a time); row totals out.
+// Per (store, group of 32 cells): sort_rows.
 __global__ void __launch_bounds__(1024) k_sort_rows(const Disc* __restrict__ discs, Ctl* __restrict__ ctl, int buf,
                                                     unsigned* __restrict__ hist, const long long* __restrict__ hoff,
                                                     unsigned* __restrict__ tot) {
     grid_dep_sync();
-    __shared__ unsigned s_sum[32][33];
     const int seg = blockIdx.y, d = seg >> 1, sp = seg & 1;
     const int N = discs[d].N;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int c = blockIdx.x * 32 + lane;
     if (blockIdx.x * 32 >= N) return;
     const unsigned Ts = (unsigned)sort_tiles(chunks_of(ctl->lay[d][sp][buf], ctl->count[d][sp], discs[d].chunk),
                                              discs[d].chunk);
-    unsigned* H = hist + hoff[seg];
-    const unsigned per = (Ts + 31) / 32, t0 = min(Ts, warp * per), t1 = min(Ts, t0 + per);
-    unsigned sum = 0;
-    if (c < N) {
-#pragma unroll 8
-        for (unsigned t = t0; t < t1; ++t) sum += H[(size_t)t * N + c];
-    }
-    s_sum[warp][lane] = sum;
-    __syncthreads();
-    unsigned pre = 0;
-    for (int w = 0; w < warp; ++w) pre += s_sum[w][lane];
-    if (warp == 31 && c < N) tot[(long long)seg * MAXN + c] = pre + sum;
-    if (c < N)
-        for (unsigned t = t0; t < t1; t += 8) {  // eight loads in flight
-            unsigned v[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) v[q] = t + q < t1 ? H[(size_t)(t + q) * N + c] : 0u;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                if (t + q < t1) H[(size_t)(t + q) * N + c] = pre;
-                pre += v[q];
-            }
-        }
-    // the last CTA of the store turns the row totals into the first slot of every cell
-    __shared__ int s_last;
-    if (warp == 31) __threadfence();  // this CTA's totals, before its count
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const unsigned prev = atomicAdd(&ctl->sort_rows_done[d][sp], 1u);
-        s_last = prev == (unsigned)((N + 31) / 32 - 1);
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    cells_scan(tot + (long long)seg * MAXN, N);
-    if (threadIdx.x == 0) ctl->sort_rows_done[d][sp] = 0;
+    sort_rows(hist + hoff[seg], Ts, N, tot + (long long)seg * MAXN, &ctl->sort_rows_done[d][sp]);
 }
 
 template <typename T>
