@@ -585,8 +585,12 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* mb, unsigned parit
 // E_{c+1} - E_c), the histograms (`sets` 2: both species at once, 5 + 3 arrays; 1: one species at a
 // time, 5 arrays) and their windows, per warp two staging buffers of one chunk (records, then cells) and its candidate
 // queue, per store its layout, per species the chunk prefix over the discharges.
-struct StoreSnap {
-    int K, chunks, M, D0, n;
+struct alignas(16) StoreSnap {
+    int K, M, D0, n;
+    const int* start;  // of the input buffer
+    const void* rec;
+    const int32_t* cell;
+    long long pad_;
 };
 template <typename T, int PPT>
 __host__ __device__ constexpr unsigned sweep_stage_bytes() {  // one buffer of one warp
@@ -703,7 +707,8 @@ __global__ void __launch_bounds__(sweep_max_threads<T>(), 1)
             ch = discs[d].ralloc[sp];
             if (blockIdx.x == 0) atomicOr(&s_err, ERR_CAPACITY);
         }
-        s_store[s] = StoreSnap{L.K, (int)ch, (int)L.M, (int)L.D0, (int)n};
+        const Seg<T>& G = segs_of<T>(discs[d])[sp];
+        s_store[s] = StoreSnap{L.K, (int)L.M, (int)L.D0, (int)n, G.start, G.p[in_buf], G.c[in_buf], 0};
         if (blockIdx.x == 0) ctl->chunks_in[d][sp] = (int)ch;  // read by the post-sweep grid
         s_pre[sp * (n_disc + 1) + d + 1] = (int)ch;
         if (d == 0) s_pre[sp * (n_disc + 1)] = 0;
@@ -787,12 +792,11 @@ __global__ void __launch_bounds__(sweep_max_threads<T>(), 1)
             warp_range(pf_s, pf_k, pf_end);
         }
         pf_b ^= 1;
-        const StoreSnap ss = s_store[pf_s];
-        const Seg<T>& G = n_disc == 1 ? s_seg[pf_s] : segs_of<T>(discs[pf_s >> 1])[pf_s & 1];
+        const StoreSnap& ss = s_store[pf_s];
         unsigned src;
         if (pf_k < ss.K) {
             src = (unsigned)pf_k * CHUNK;
-            const int* st = G.start + pf_k;
+            const int* st = ss.start + pf_k;
             pf_base = __ldcg(st);
             pf_stop = __ldcg(st + 1);
         } else {
@@ -806,14 +810,15 @@ __global__ void __launch_bounds__(sweep_max_threads<T>(), 1)
             unsigned long long* mb = &s_mbar[warp][pf_b];
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // earlier reads and writes of the buffer
             mbar_expect(mb, REC_BYTES + CELL_BYTES);
-            bulk_g2s(buf, reinterpret_cast<const R*>(G.p[in_buf]) + src, REC_BYTES, mb);
-            bulk_g2s(buf + REC_BYTES, G.c[in_buf] + src, CELL_BYTES, mb);
+            bulk_g2s(buf, static_cast<const R*>(ss.rec) + src, REC_BYTES, mb);
+            bulk_g2s(buf + REC_BYTES, ss.cell + src, CELL_BYTES, mb);
         }
     };
     prefetch_next();
 
     const unsigned lt = (1u << lane) - 1u;
-    int err = 0;
+    int err = 0, cur_d = -1;
+    unsigned sumA = 0, sumB = 0, sumS = 0;  // survivors and newborns since the last add to the slice sums
     unsigned carry = 0, carry_q = 0xFFFFFFFFu;  // candidate bits of the last call of the warp's previous chunk
 
     // One warp's chunk of the store of species SP (see above).
@@ -947,7 +952,7 @@ __global__ void __launch_bounds__(sweep_max_threads<T>(), 1)
                 const unsigned mA = __ballot_sync(FULL, alive);
                 bool see = false;
                 Part<T> Pse{};
-                if (__any_sync(FULL, in && !alive) && in && !alive) {
+                if (mA != (cnt - 32 * k < 32 ? (1u << (cnt - 32 * k)) - 1u : FULL) && in && !alive) {
                     if (!valid || !(s == s)) err |= ERR_NONFINITE;  // a corrupt cell index is dropped too
                     if (valid) {
                         const int side = s >= (T)0 ? 1 : 0;
@@ -966,15 +971,23 @@ __global__ void __launch_bounds__(sweep_max_threads<T>(), 1)
                 }
             }
         }
+        sumA += offA - obase;
+        sumB += offB - obase;
+        sumS += offS - obase;
         if (lane == 0) {
-            const unsigned a = offA - obase, b = offB - obase, c = offS - obase;
-            S.cnt_main[cs] = (int)a;
-            S.cnt_birth[cs] = (int)b;
-            if (SP == 0) S.cnt_same[cs] = (int)c;
-            unsigned* sl = S.slice_tot + s_par * S.slice_stride + 3 * (cs / SLICE);
-            if (a) atomicAdd(&sl[0], a);
-            if (b) atomicAdd(&sl[1], b);
-            if (SP == 0 && c) atomicAdd(&sl[2], c);
+            S.cnt_main[cs] = (int)(offA - obase);
+            S.cnt_birth[cs] = (int)(offB - obase);
+            if (SP == 0) S.cnt_same[cs] = (int)(offS - obase);
+        }
+        // the slice sums once per run of the warp's chunks in a slice
+        if (pf_s != 2 * cur_d + SP || (cs + 1) % SLICE == 0) {
+            if (lane == 0) {
+                unsigned* sl = S.slice_tot + s_par * S.slice_stride + 3 * (cs / SLICE);
+                if (sumA) atomicAdd(&sl[0], sumA);
+                if (sumB) atomicAdd(&sl[1], sumB);
+                if (sumS) atomicAdd(&sl[2], sumS);
+            }
+            sumA = sumB = sumS = 0;
         }
     };
 
@@ -1023,7 +1036,7 @@ __global__ void __launch_bounds__(sweep_max_threads<T>(), 1)
     };
 
     const int flush_rounds = max(1, flush_particles<T>() / (NW * CHUNK));
-    int cur_d = -1, cur_sp = 0;
+    int cur_sp = 0;
     for (int s = next_store(-1); s < n_store; s = next_store(s)) {
         const int d = s >> 1, sp = s & 1;
         if (cur_d >= 0 && (d != cur_d || sets == 1)) {
@@ -1041,9 +1054,9 @@ __global__ void __launch_bounds__(sweep_max_threads<T>(), 1)
                 const int2 g = s_range[2 * d + q];
                 int w0 = NO_WIN;
                 if (g.y - g.x >= WIN_CHUNKS) {
-                    const StoreSnap ss = s_store[2 * d + q];
+                    const StoreSnap& ss = s_store[2 * d + q];
                     auto first_cell = [&](int k) {
-                        return __ldcg(s_seg[q].c[in_buf] +
+                        return __ldcg(ss.cell +
                                       (k < ss.K ? (unsigned)k * CHUNK : (unsigned)(ss.D0 + (k - ss.K) * CHUNK)));
                     };
                     const int a = first_cell(g.x), b = first_cell(g.y - 1);
@@ -1058,10 +1071,11 @@ __global__ void __launch_bounds__(sweep_max_threads<T>(), 1)
         cur_sp = sp;
         carry_q = 0xFFFFFFFFu;
         const int rounds = (s_range[s].y - s_range[s].x + NW - 1) / NW;  // chunks of this store a warp has at most
-        for (int r = 0; r < rounds; ++r) {
-            if (r > 0 && r % flush_rounds == 0) {
+        for (int r = 0, f = flush_rounds; r < rounds; ++r) {
+            if (f-- == 0) {
                 flush(cur_sp);
                 clear();
+                f = flush_rounds - 1;
             }
             if (pf_s != s) continue;
             const unsigned cs = (unsigned)pf_k;
