@@ -205,10 +205,14 @@ __device__ __forceinline__ void energy_add(const Hist& h, unsigned long long* Qg
         atomicAdd(a + 3 * st, Et & 0x1FFFFu);
         atomicAdd(a + 4 * st, Eh & 0x1FFFFu);
     }
-    if (__any_sync(FULL, on && (Et >> 17)) && on && (Et >> 17)) {
-        const unsigned long long ht = Et >> 17, hh = Eh >> 17;
-        atomicAdd(&Qg[c], (ht - hh) << 17);
-        if (hh) atomicAdd(&Qg[c + 1], hh << 17);
+    const bool high = on && (Et >> 17);
+    if (__any_sync(FULL, high)) {
+        if (high) {
+            const unsigned long long ht = Et >> 17, hh = Eh >> 17;
+            atomicAdd(&Qg[c], (ht - hh) << 17);
+            if (hh) atomicAdd(&Qg[c + 1], hh << 17);
+        }
+        __syncwarp();  // keeps this a branch: as predicated instructions the rare part costs every row 17 of them
     }
 }
 
@@ -950,25 +954,28 @@ __global__ void __launch_bounds__(sweep_max_threads<T>(), 1)
                 T fn, s;
                 const bool alive = drift_fast(N, dtdx, c, r.x, vz, cn, fn, s) && valid;
                 const unsigned mA = __ballot_sync(FULL, alive);
-                bool see = false;
-                Part<T> Pse{};
-                if (mA != (cnt - 32 * k < 32 ? (1u << (cnt - 32 * k)) - 1u : FULL) && in && !alive) {
-                    if (!valid || !(s == s)) err |= ERR_NONFINITE;  // a corrupt cell index is dropped too
-                    if (valid) {
-                        const int side = s >= (T)0 ? 1 : 0;
-                        atomicAdd(&s_cnt[CNT_ABS + 2 * SP + side], 1u);
-                        if (SP == 1 && S.has_see)
-                            see = emit_see<T>(S, S.Dother + s_dpar * (N + 1), (uint32_t)base + i, rs, side, Pse, s_cnt);
+                if (mA != (cnt - 32 * k < 32 ? (1u << (cnt - 32 * k)) - 1u : FULL)) {  // some left the gap
+                    bool see = false;
+                    Part<T> Pse{};
+                    if (in && !alive) {
+                        if (!valid || !(s == s)) err |= ERR_NONFINITE;  // a corrupt cell index is dropped too
+                        if (valid) {
+                            const int side = s >= (T)0 ? 1 : 0;
+                            atomicAdd(&s_cnt[CNT_ABS + 2 * SP + side], 1u);
+                            if (SP == 1 && S.has_see)
+                                see = emit_see<T>(S, S.Dother + s_dpar * (N + 1), (uint32_t)base + i, rs, side, Pse, s_cnt);
+                        }
                     }
+                    if (SP == 1) {
+                        const unsigned mB = __ballot_sync(FULL, see);
+                        if (see) store_rec<T>(S.bc, S.bp, offB + __popc(mB & lt), Pse);
+                        offB += __popc(mB);
+                    }
+                    __syncwarp();
                 }
                 warp_dep<SP == 1>(h, alive ? cn : -1, cic_F(fn), lane);
                 if (alive) store_rec<T>(cout, pout, offA + __popc(mA & lt), Part<T>{cn, fn, r.y, r.z, vz});
                 offA += __popc(mA);
-                if (SP == 1 && S.has_see) {
-                    const unsigned mB = __ballot_sync(FULL, see);
-                    if (see) store_rec<T>(S.bc, S.bp, offB + __popc(mB & lt), Pse);
-                    offB += __popc(mB);
-                }
             }
         }
         sumA += offA - obase;
