@@ -3,6 +3,7 @@
 // sequence (sweep -> finalize -> periodic sort), optionally replayed from CUDA
 // graphs of one rf period.
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -59,7 +60,8 @@ struct pic_ctx {
     int max_slices = 0;  // slices of sweep chunks of the largest store
     void* stage = nullptr;  // device staging of state transfers
     size_t stage_bytes = 0;
-    void* h_pin = nullptr;  // pinned host scratch for read-backs (one stream sync per call)
+    void* h_pin = nullptr;  // pinned, mapped host scratch for read-backs (one stream sync per call)
+    void* h_pin_dev = nullptr;  // its device address
     size_t h_pin_bytes = 0;
     std::string err;
     pic_counters cnt_at_reset[MAXD];
@@ -901,9 +903,10 @@ static pic_status pinned(pic_ctx* ctx, size_t bytes) {
     bytes = std::max(bytes, (size_t)1 << 16);
     CK(cudaStreamSynchronize(ctx->stream), "synchronize");
     if (ctx->h_pin) cudaFreeHost(ctx->h_pin);
-    ctx->h_pin = nullptr;
+    ctx->h_pin = ctx->h_pin_dev = nullptr;
     ctx->h_pin_bytes = 0;
-    CK(cudaMallocHost(&ctx->h_pin, bytes), "pinned scratch");
+    CK(cudaHostAlloc(&ctx->h_pin, bytes, cudaHostAllocMapped), "pinned scratch");
+    CK(cudaHostGetDevicePointer(&ctx->h_pin_dev, ctx->h_pin, 0), "pinned scratch");
     ctx->h_pin_bytes = bytes;
     return PIC_OK;
 }
@@ -923,16 +926,24 @@ extern "C" pic_status pic_get_count(pic_ctx* ctx, int32_t d, int32_t sp, int64_t
 static size_t pad16(size_t b) { return (b + 15) / 16 * 16; }
 
 // Device staging of a state transfer: the cells and the four real arrays, each starting on a
-// 16-byte boundary (the pack / unpack kernels then move whole 16-byte groups), and an error word.
+// 16-byte boundary (the pack / unpack kernels then move whole 16-byte groups). With an eighth to spare
+// where there is room, so that a store that grows from call to call does not allocate on each
+// (cudaFree and cudaMalloc: 115 us).
 static pic_status staging(pic_ctx* ctx, long long n) {
     const size_t r = ctx->fp64 ? 8 : 4;
-    const size_t need = pad16((size_t)n * 4) + 4 * pad16((size_t)n * r) + 64;
+    size_t need = pad16((size_t)n * 4) + 4 * pad16((size_t)n * r);
     if (ctx->stage_bytes >= need) return PIC_OK;
     CK(cudaStreamSynchronize(ctx->stream), "synchronize");
     if (ctx->stage) cudaFree(ctx->stage);
     ctx->stage = nullptr;
     ctx->stage_bytes = 0;
-    CK(cudaMalloc(&ctx->stage, need), "staging");
+    if (cudaMalloc(&ctx->stage, need + need / 8) == cudaSuccess) {
+        need += need / 8;
+    } else {
+        cudaGetLastError();  // no room to spare: the size itself
+        ctx->stage = nullptr;
+        CK(cudaMalloc(&ctx->stage, need), "staging");
+    }
     ctx->stage_bytes = need;
     return PIC_OK;
 }
@@ -970,9 +981,9 @@ extern "C" pic_status pic_get_state(pic_ctx* ctx, int32_t d, int32_t sp, int64_t
         const int grid = std::max(1, (int)std::min<long long>(ctx->num_sms * 8, (cap + 255) / 256));
         void* const v[4] = {hm[1], hm[2], hm[3], hm[4]};
         CK(launch_unpack_state(ctx->fp64, ctx->d_discs, ctx->d_ctl, d, sp, ctx->cur, cap,
-                               static_cast<int32_t*>(hm[0]), v, grid, ctx->stream),
+                               static_cast<int32_t*>(hm[0]), v, static_cast<long long*>(ctx->h_pin_dev), grid,
+                               ctx->stream),
            "state gather");
-        CK(cudaMemcpyAsync(hn, &ctx->d_ctl->count[d][sp], 8, cudaMemcpyDeviceToHost, ctx->stream), "count");
         CK(cudaStreamSynchronize(ctx->stream), "state copy");
         if (n_out) *n_out = *hn;
         if (*hn > cap) return fail(ctx, PIC_ERR_ARG, "host buffer too small");
@@ -993,7 +1004,8 @@ extern "C" pic_status pic_get_state(pic_ctx* ctx, int32_t d, int32_t sp, int64_t
     const size_t sr = pad16((size_t)n * r);
     {
         void* const v[4] = {sv, sv + sr, sv + 2 * sr, sv + 3 * sr};
-        CK(launch_unpack_state(ctx->fp64, ctx->d_discs, ctx->d_ctl, d, sp, ctx->cur, n, sc, v, grid, ctx->stream),
+        CK(launch_unpack_state(ctx->fp64, ctx->d_discs, ctx->d_ctl, d, sp, ctx->cur, n, sc, v, nullptr, grid,
+                               ctx->stream),
            "state gather");
     }
     if (c) CK(cudaMemcpyAsync(c, sc, 4 * (size_t)n, cudaMemcpyDeviceToHost, ctx->stream), "state c");
@@ -1011,53 +1023,53 @@ extern "C" pic_status pic_set_state(pic_ctx* ctx, int32_t d, int32_t sp, int64_t
     const Disc& D = ctx->hd[d];
     if (n > D.cap[sp]) return fail(ctx, PIC_ERR_CAPACITY, "state larger than capacity");
     const size_t r = ctx->fp64 ? 8 : 4;
-    pic_status s = staging(ctx, n > 0 ? n : 1);
+    pic_status s = pinned(ctx, 64);
     if (s != PIC_OK) return s;
-    int32_t* sc = static_cast<int32_t*>(ctx->stage);
-    unsigned char* sv = static_cast<unsigned char*>(ctx->stage) + pad16((size_t)n * 4);
-    const size_t sr = pad16((size_t)n * r);
-    unsigned* bad = reinterpret_cast<unsigned*>(static_cast<unsigned char*>(ctx->stage) + ctx->stage_bytes - 64);
-    CK(cudaMemsetAsync(bad, 0, sizeof(unsigned), ctx->stream), "state check");
+    const void* src[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     if (n) {
-        const int grid = std::max(1, std::min(ctx->num_sms * 8, (int)((n + 255) / 256)));
-        const void* hm[5] = {mapped(c), mapped(f), mapped(vx), mapped(vy), mapped(vz)};
-        if (hm[0] && hm[1] && hm[2] && hm[3] && hm[4]) {  // mapped: the pack kernel reads them directly
-            const void* const v[4] = {hm[1], hm[2], hm[3], hm[4]};
-            CK(launch_pack_state(ctx->fp64, ctx->d_discs, d, sp, ctx->cur, n, static_cast<const int32_t*>(hm[0]), v,
-                                 bad, grid, ctx->stream),
-               "state pack");
-        } else {
-            CK(cudaMemcpyAsync(sc, c, 4 * (size_t)n, cudaMemcpyHostToDevice, ctx->stream), "state c");
-            const void* ins[4] = {f, vx, vy, vz};
-            for (int q = 0; q < 4; ++q)
-                CK(cudaMemcpyAsync(sv + q * sr, ins[q], r * (size_t)n, cudaMemcpyHostToDevice,
-                                   ctx->stream),
-                   "state p");
-            const void* const v[4] = {sv, sv + sr, sv + 2 * sr, sv + 3 * sr};
-            CK(launch_pack_state(ctx->fp64, ctx->d_discs, d, sp, ctx->cur, n, sc, v, bad, grid, ctx->stream),
-               "state pack");
+        const void* in[5] = {c, f, vx, vy, vz};
+        bool direct = true;
+        for (int q = 0; q < 5 && direct; ++q) direct = (src[q] = mapped(in[q])) != nullptr;
+        if (!direct) {  // else the pack kernel reads the mapped arrays directly
+            s = staging(ctx, n);
+            if (s != PIC_OK) return s;
+            unsigned char* p = static_cast<unsigned char*>(ctx->stage);
+            for (int q = 0; q < 5; ++q) {
+                const size_t bytes = (q ? r : 4) * (size_t)n;
+                CK(cudaMemcpyAsync(p, in[q], bytes, cudaMemcpyHostToDevice, ctx->stream), "state copy");
+                src[q] = p;
+                p += pad16(bytes);
+            }
         }
     }
-    // count and dense layout on the device (a rejected upload leaves an empty store), then one
+    // the kernel also sets count and dense layout (a rejected upload leaves an empty store); one
     // synchronisation for the check word
-    CK(launch_finish_upload(ctx->d_discs, ctx->d_ctl, d, sp, n, bad, ctx->cur, ctx->stream), "state finish");
-    s = pinned(ctx, 64);
-    if (s != PIC_OK) return s;
-    unsigned* hbad = static_cast<unsigned*>(ctx->h_pin);
-    CK(cudaMemcpyAsync(hbad, bad, sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->stream), "state check");
+    const int grid = std::max(1, (int)std::min<long long>(ctx->num_sms * 8, (n + 255) / 256));
+    const void* const v[4] = {src[1], src[2], src[3], src[4]};
+    CK(launch_pack_state(ctx->fp64, ctx->d_discs, ctx->d_ctl, d, sp, ctx->cur, n, static_cast<const int32_t*>(src[0]), v,
+                         static_cast<unsigned*>(ctx->h_pin_dev), grid, ctx->stream),
+       "state pack");
     CK(cudaStreamSynchronize(ctx->stream), "state copy");
-    if (*hbad) return fail(ctx, PIC_ERR_ARG, "cell index out of range");
+    if (*static_cast<const unsigned*>(ctx->h_pin)) return fail(ctx, PIC_ERR_ARG, "cell index out of range");
     return PIC_OK;
 }
 
 extern "C" pic_status pic_get_field(pic_ctx* ctx, int32_t d, void* E, double* E64, double* phi) {
     if (bad_d(ctx, d)) return PIC_ERR_ARG;
-    CK(cudaStreamSynchronize(ctx->stream), "synchronize");
     const Disc& D = ctx->hd[d];
-    const size_t N1 = (size_t)D.N + 1, r = ctx->fp64 ? 8 : 4;
-    if (E) CK(cudaMemcpy(E, D.E, r * N1, cudaMemcpyDeviceToHost), "field");
-    if (E64) CK(cudaMemcpy(E64, D.E64, 8 * N1, cudaMemcpyDeviceToHost), "field64");
-    if (phi) CK(cudaMemcpy(phi, D.phi, 8 * N1, cudaMemcpyDeviceToHost), "phi");
+    const size_t N1 = (size_t)D.N + 1, r = ctx->fp64 ? 8 : 4, o_phi = 8 * N1, o_E = 16 * N1;
+    pic_status s = pinned(ctx, o_E + r * N1);
+    if (s != PIC_OK) return s;
+    Gather g{};
+    g.add(D.E64, 0, 8 * N1);
+    g.add(D.phi, o_phi, 8 * N1);
+    g.add(D.E, o_E, r * N1);
+    CK(launch_gather(g, ctx->h_pin_dev, ctx->num_sms, ctx->stream), "field");
+    CK(cudaStreamSynchronize(ctx->stream), "field");
+    const unsigned char* h = static_cast<const unsigned char*>(ctx->h_pin);
+    if (E) std::memcpy(E, h + o_E, r * N1);
+    if (E64) std::memcpy(E64, h, 8 * N1);
+    if (phi) std::memcpy(phi, h + o_phi, 8 * N1);
     return PIC_OK;
 }
 
@@ -1171,10 +1183,15 @@ extern "C" pic_status pic_moments(pic_ctx* ctx, int32_t d, pic_moments_t* out) {
     const Disc& D = ctx->hd[d];
     const int N = D.N;
     const size_t N1 = (size_t)N + 1;
-    // every read-back of the call into pinned memory, one synchronisation: the four exact
-    // accumulators (one block), the control block, the counters, the last J(t) and the last
-    // period's current amplitude
-    const size_t acc = 16 * N1, o_ctl = 4 * acc, o_cnt = o_ctl + ((sizeof(Ctl) + 15) / 16) * 16;
+    // every read-back of the call into pinned memory by one launch, one synchronisation: the four exact
+    // accumulators (one block), this discharge's words of the control block, the counters, the last J(t)
+    // and the last period's current amplitude
+    struct Words {
+        long long count[2], acc_steps;
+        double E0_last;
+        int error, pad;
+    };
+    const size_t acc = 16 * N1, o_ctl = 4 * acc, o_cnt = o_ctl + sizeof(Words);
     const size_t o_j = o_cnt + 8 * NCNT;
     pic_status s = pinned(ctx, o_j + 3 * sizeof(double));
     if (s != PIC_OK) return s;
@@ -1183,18 +1200,20 @@ extern "C" pic_status pic_moments(pic_ctx* ctx, int32_t d, pic_moments_t* out) {
     const long long done = spp > 0 ? ctx->step / spp : 0;
     double* hj = reinterpret_cast<double*>(h + o_j);
     hj[0] = hj[1] = hj[2] = 0.0;
-    CK(cudaMemcpyAsync(h, D.acc_D[0], 4 * acc, cudaMemcpyDeviceToHost, ctx->stream), "moments");
-    CK(cudaMemcpyAsync(h + o_ctl, ctx->d_ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, ctx->stream), "moments");
-    CK(cudaMemcpyAsync(h + o_cnt, D.cnt, 8 * NCNT, cudaMemcpyDeviceToHost, ctx->stream), "moments");
+    Gather g{};
+    g.add(D.acc_D[0], 0, 4 * acc);
+    g.add(ctx->d_ctl->count[d], o_ctl + offsetof(Words, count), 16);
+    g.add(&ctx->d_ctl->acc_steps[d], o_ctl + offsetof(Words, acc_steps), 8);
+    g.add(&ctx->d_ctl->E0_last[d], o_ctl + offsetof(Words, E0_last), 8);
+    g.add(&ctx->d_ctl->error, o_ctl + offsetof(Words, error), 4);
+    g.add(D.cnt, o_cnt, 8 * NCNT);
     if (ctx->step > 0) {
-        CK(cudaMemcpyAsync(hj, D.J_hist + 2 * ((ctx->step - 1) % D.jh), 2 * sizeof(double), cudaMemcpyDeviceToHost,
-                           ctx->stream), "current");
-        if (done > 0 && D.jtab)
-            CK(cudaMemcpyAsync(hj + 2, D.J_amp + (done - 1) % PERIOD_HIST, sizeof(double), cudaMemcpyDeviceToHost,
-                               ctx->stream), "current amplitude");
+        g.add(D.J_hist + 2 * ((ctx->step - 1) % D.jh), o_j, 2 * sizeof(double));
+        if (done > 0 && D.jtab) g.add(D.J_amp + (done - 1) % PERIOD_HIST, o_j + 16, sizeof(double));
     }
+    CK(launch_gather(g, ctx->h_pin_dev, ctx->num_sms, ctx->stream), "moments");
     CK(cudaStreamSynchronize(ctx->stream), "moments");
-    const Ctl& hc = *reinterpret_cast<const Ctl*>(h + o_ctl);
+    const Words& hc = *reinterpret_cast<const Words*>(h + o_ctl);
     if (hc.error & ERR_TIMEOUT) return fail(ctx, PIC_ERR_TIMEOUT, "a bounded device-side wait timed out");
     if (hc.error & ERR_CAPACITY) return fail(ctx, PIC_ERR_CAPACITY, "particle or birth buffer capacity exceeded");
     if (hc.error & ERR_NONFINITE) return fail(ctx, PIC_ERR_NONFINITE, "non-finite particle coordinate");
@@ -1202,7 +1221,7 @@ extern "C" pic_status pic_moments(pic_ctx* ctx, int32_t d, pic_moments_t* out) {
     const unsigned __int128* iD1 = reinterpret_cast<const unsigned __int128*>(h + acc);
     const unsigned __int128* iQ = reinterpret_cast<const unsigned __int128*>(h + 2 * acc);
     const unsigned __int128* iP = reinterpret_cast<const unsigned __int128*>(h + 3 * acc);
-    const long long steps = hc.acc_steps[d];
+    const long long steps = hc.acc_steps;
     const double dx = D.dx, ns = steps > 0 ? (double)steps : 1.0;
     for (int j = 0; j <= N; ++j) {
         const double Vj = (j == 0 || j == N) ? 0.5 * dx : dx;
@@ -1214,14 +1233,14 @@ extern "C" pic_status pic_moments(pic_ctx* ctx, int32_t d, pic_moments_t* out) {
     pic_counters c;
     parse_counters(reinterpret_cast<const unsigned long long*>(h + o_cnt), &c);
     out->steps = steps;
-    out->count[0] = hc.count[d][0];
-    out->count[1] = hc.count[d][1];
+    out->count[0] = hc.count[0];
+    out->count[1] = hc.count[1];
     for (int a = 0; a < 2; ++a)
         for (int b = 0; b < 2; ++b) {
             out->absorbed[a][b] = (double)(c.absorbed[a][b] - ctx->cnt_at_reset[d].absorbed[a][b]);
             out->flux[a][b] = steps > 0 ? out->absorbed[a][b] * D.w[a] / ((double)steps * D.dt) : 0.0;
         }
-    out->surface_charge = 8.8541878128e-12 * hc.E0_last[d];
+    out->surface_charge = 8.8541878128e-12 * hc.E0_last;
     // rf periods, the steady-state criterion on the per-period mean counts, J(t)
     out->periods_done = done;
     out->steady_period = -1;
@@ -1399,10 +1418,12 @@ extern "C" pic_status pic_diagnostics(pic_ctx* ctx, int32_t d, double* E, double
     pic_status s = pinned(ctx, o_n + 16);
     if (s != PIC_OK) return s;
     unsigned char* h = static_cast<unsigned char*>(ctx->h_pin);
-    CK(cudaMemcpyAsync(h, D.dg, o_E, cudaMemcpyDeviceToHost, ctx->stream), "diagnostics");
-    CK(cudaMemcpyAsync(h + o_E, D.dg_E, 8 * N1, cudaMemcpyDeviceToHost, ctx->stream), "diagnostics");
-    CK(cudaMemcpyAsync(h + o_h, D.dg_eedf, 8 * (size_t)bins, cudaMemcpyDeviceToHost, ctx->stream), "diagnostics");
-    CK(cudaMemcpyAsync(h + o_n, D.dg_n, 16, cudaMemcpyDeviceToHost, ctx->stream), "diagnostics");
+    Gather g{};
+    g.add(D.dg, 0, o_E);
+    g.add(D.dg_E, o_E, 8 * N1);
+    g.add(D.dg_eedf, o_h, 8 * (size_t)bins);
+    g.add(D.dg_n, o_n, 16);
+    CK(launch_gather(g, ctx->h_pin_dev, ctx->num_sms, ctx->stream), "diagnostics");
     CK(cudaStreamSynchronize(ctx->stream), "diagnostics");
     const long long* A = reinterpret_cast<const long long*>(h);  // exact sums, two's complement
     const long long *aD = A + DG_D * N1, *aU = A + DG_U * N1, *aV = A + DG_V * N1, *aW = A + DG_W * N1,

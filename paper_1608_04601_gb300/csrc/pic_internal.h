@@ -204,6 +204,22 @@ struct Ctl {
     double J_drive[MAXD];
     double period_acc[MAXD][2];   // sum of the counts over the steps of the current rf period
     unsigned sort_rows_done[MAXD][2];  // k_sort_rows CTAs finished, per store (reset by the last)
+    unsigned up_bad, up_done;  // state upload: cells out of range, CTAs finished (both 0 between uploads)
+};
+
+// Read-back of several device arrays into one pinned host block: part q goes to byte off[q]; sizes in
+// 4-byte words, end[q] the words of the parts up to and including q.
+constexpr int GATHER_MAX = 8;
+struct Gather {
+    int n;
+    const void* src[GATHER_MAX];
+    unsigned off[GATHER_MAX], end[GATHER_MAX];
+    void add(const void* p, size_t at, size_t bytes) {
+        src[n] = p;
+        off[n] = (unsigned)at;
+        end[n] = (n ? end[n - 1] : 0u) + (unsigned)(bytes / 4);
+        ++n;
+    }
 };
 
 // Chunks of a store with layout L and count n.

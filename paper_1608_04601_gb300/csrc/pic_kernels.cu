@@ -2190,13 +2190,17 @@ __device__ __forceinline__ bool aligned16(const void* a, const void* b, const vo
 }
 
 // State upload: SoA arrays (device staging, or the caller's mapped pinned host arrays) -> the
-// store's records; cells outside [0, N) are counted in *bad. With 16-byte aligned arrays each
+// store's records; cells outside [0, N) are counted. With 16-byte aligned arrays each
 // thread reads whole 16-byte groups (over the host link, wide loads keep more bytes in flight
-// per thread), the ragged tail one by one.
+// per thread), the ragged tail one by one. The last CTA sets the store: n particles, or none if a cell was
+// out of range, dense in buffer buf; the count of such cells goes to *bad_out (mapped host memory). Bounded by
+// the host link (1e6 particles, 20 MB: 99 us, the copy engine takes 97); the layout, the check word and its way
+// back in this launch, and no staging for mapped arrays: a call of 1e6 particles 134 (250 where the
+// staging had grown) -> 121 us.
 template <typename T>
-__global__ void k_pack_state(const Disc* __restrict__ discs, int d, int sp, int buf, long long n,
+__global__ void k_pack_state(const Disc* __restrict__ discs, Ctl* __restrict__ ctl, int d, int sp, int buf, long long n,
                              const int32_t* __restrict__ c, const T* __restrict__ f, const T* __restrict__ vx,
-                             const T* __restrict__ vy, const T* __restrict__ vz, unsigned* __restrict__ bad) {
+                             const T* __restrict__ vy, const T* __restrict__ vz, unsigned* __restrict__ bad_out) {
     typedef XferVec<T> X;
     const Disc& D = discs[d];
     const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, nt = (long long)gridDim.x * blockDim.x;
@@ -2222,7 +2226,17 @@ __global__ void k_pack_state(const Disc* __restrict__ discs, int d, int sp, int 
         nbad += (unsigned)ci >= (unsigned)D.N;
         store_rec<T>(D.c[buf][sp], D.p[buf][sp], (unsigned)i, Part<T>{ci, f[i], vx[i], vy[i], vz[i]});
     }
-    if (nbad) atomicAdd(bad, nbad);
+    if (nbad) atomicAdd(&ctl->up_bad, nbad);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&ctl->up_done, 1u) == gridDim.x - 1) {
+        __threadfence();
+        const unsigned all_bad = atomicExch(&ctl->up_bad, 0u);
+        ctl->up_done = 0;
+        ctl->count[d][sp] = all_bad ? 0 : n;
+        ctl->lay[d][sp][buf] = Lay{0, 0, 0, 0};
+        *bad_out = all_bad;
+    }
 }
 
 // Position i of the state in the store: regions (binary search of the start table; empty regions
@@ -2240,15 +2254,16 @@ __device__ __forceinline__ long long state_slot(const Lay& L, const int* st, int
 
 // State download: the store, read through its layout -> SoA arrays (device staging, or the
 // caller's mapped pinned host arrays; null outputs are skipped). The count comes from the control
-// block; above cap nothing is written. With 16-byte aligned outputs each thread writes whole
-// 16-byte groups.
+// block and goes to *n_out if that is not null; above cap nothing else is written. With 16-byte aligned
+// outputs each thread writes whole 16-byte groups.
 template <typename T>
 __global__ void k_unpack_state(const Disc* __restrict__ discs, const Ctl* __restrict__ ctl, int d, int sp, int buf,
                                long long cap, int32_t* __restrict__ c, T* __restrict__ f, T* __restrict__ vx,
-                               T* __restrict__ vy, T* __restrict__ vz) {
+                               T* __restrict__ vy, T* __restrict__ vz, long long* __restrict__ n_out) {
     typedef XferVec<T> X;
     const Disc& D = discs[d];
     const long long n = ctl->count[d][sp];
+    if (n_out && blockIdx.x == 0 && threadIdx.x == 0) *n_out = n;
     if (n > cap) return;
     const Lay L = ctl->lay[d][sp][buf];
     const int* st = D.start[sp];
@@ -2284,13 +2299,20 @@ __global__ void k_unpack_state(const Disc* __restrict__ discs, const Ctl* __rest
     }
 }
 
-// End of a state upload (one thread): the store holds n particles, or none if the pack kernel found a
-// cell out of range, dense in buffer buf.
-__global__ void k_finish_upload(const Disc* __restrict__ discs, Ctl* __restrict__ ctl, int d, int sp, long long n,
-                                const unsigned* __restrict__ bad, int buf) {
-    ctl->count[d][sp] = *bad ? 0 : n;
-    ctl->lay[d][sp][buf] = Lay{0, 0, 0, 0};
+// Several device arrays into one block of mapped host memory. A read-back of a few 10 KB is bounded by its
+// launches: one of these in place of three to five copies (each about 8 us of engine and queue) takes
+// pic_moments from 90 to 74 us at 512 cells (16 us of launch and copy; the rest is the host's
+// conversion of the exact sums), a batch of 64 discharges' by 1.5 ms.
+__global__ void __launch_bounds__(256) k_gather(const Gather g, unsigned* __restrict__ out) {
+    const unsigned words = g.end[g.n - 1];
+    for (unsigned i = blockIdx.x * 256 + threadIdx.x; i < words; i += gridDim.x * 256) {
+        int q = 0;
+        while (i >= g.end[q]) ++q;
+        const unsigned k = i - (q ? g.end[q - 1] : 0u);
+        out[g.off[q] / 4 + k] = __ldcg(static_cast<const unsigned*>(g.src[q]) + k);
+    }
 }
+
 // Every store dense in buffer buf (after a load).
 __global__ void k_set_dense(const Disc* __restrict__ discs, int n_disc, Ctl* __restrict__ ctl, int buf) {
     grid_dep_sync();
@@ -2554,36 +2576,37 @@ cudaError_t launch_repack(int fp64, const Disc* discs, int n_disc, Ctl* ctl, int
     return launch_pdl(k_repack<float>, g, dim3(256), 0, st, discs, ctl, src, dst);
 }
 
-cudaError_t launch_pack_state(int fp64, const Disc* discs, int d, int sp, int buf, long long n, const int32_t* c,
-                              const void* const v[4], unsigned* bad, int grid, cudaStream_t st) {
+cudaError_t launch_pack_state(int fp64, const Disc* discs, Ctl* ctl, int d, int sp, int buf, long long n,
+                              const int32_t* c, const void* const v[4], unsigned* bad_out, int grid, cudaStream_t st) {
     if (fp64)
-        k_pack_state<double><<<grid, 256, 0, st>>>(discs, d, sp, buf, n, c, (const double*)v[0], (const double*)v[1],
-                                                   (const double*)v[2], (const double*)v[3], bad);
+        k_pack_state<double><<<grid, 256, 0, st>>>(discs, ctl, d, sp, buf, n, c, (const double*)v[0],
+                                                   (const double*)v[1], (const double*)v[2], (const double*)v[3],
+                                                   bad_out);
     else
-        k_pack_state<float><<<grid, 256, 0, st>>>(discs, d, sp, buf, n, c, (const float*)v[0], (const float*)v[1],
-                                                  (const float*)v[2], (const float*)v[3], bad);
+        k_pack_state<float><<<grid, 256, 0, st>>>(discs, ctl, d, sp, buf, n, c, (const float*)v[0], (const float*)v[1],
+                                                  (const float*)v[2], (const float*)v[3], bad_out);
     return cudaGetLastError();
 }
 
 cudaError_t launch_unpack_state(int fp64, const Disc* discs, const Ctl* ctl, int d, int sp, int buf, long long cap,
-                                int32_t* c, void* const v[4], int grid, cudaStream_t st) {
+                                int32_t* c, void* const v[4], long long* n_out, int grid, cudaStream_t st) {
     if (fp64)
         k_unpack_state<double><<<grid, 256, 0, st>>>(discs, ctl, d, sp, buf, cap, c, (double*)v[0], (double*)v[1],
-                                                     (double*)v[2], (double*)v[3]);
+                                                     (double*)v[2], (double*)v[3], n_out);
     else
         k_unpack_state<float><<<grid, 256, 0, st>>>(discs, ctl, d, sp, buf, cap, c, (float*)v[0], (float*)v[1],
-                                                    (float*)v[2], (float*)v[3]);
+                                                    (float*)v[2], (float*)v[3], n_out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_gather(const Gather& g, void* out, int sms, cudaStream_t st) {
+    const unsigned ctas = (g.end[g.n - 1] + 255) / 256;
+    k_gather<<<ctas < (unsigned)sms ? ctas : (unsigned)sms, 256, 0, st>>>(g, static_cast<unsigned*>(out));
     return cudaGetLastError();
 }
 
 
 long long sort_tile_chunks(int chunk) { return SORT_TILE / chunk; }
-
-cudaError_t launch_finish_upload(const Disc* discs, Ctl* ctl, int d, int sp, long long n, const unsigned* bad,
-                                 int buf, cudaStream_t st) {
-    k_finish_upload<<<1, 1, 0, st>>>(discs, ctl, d, sp, n, bad, buf);
-    return cudaGetLastError();
-}
 
 // Dynamic shared memory of a k_diag launch: its node arrays and, for a sample, the EEDF (bins > 0).
 size_t diag_smem(int max_N, unsigned mask, int bins) {

@@ -34,10 +34,11 @@ cudaError_t launch_repack(int fp64, const Disc* discs, int n_disc, Ctl* ctl, int
                           cudaStream_t st);
 // state transfer: cells and the four SoA value arrays (f, vx, vy, vz), in device staging or mapped
 // pinned host memory; a null output array of the unpack is skipped
-cudaError_t launch_pack_state(int fp64, const Disc* discs, int d, int sp, int buf, long long n, const int32_t* c,
-                              const void* const v[4], unsigned* bad, int grid, cudaStream_t st);
+cudaError_t launch_pack_state(int fp64, const Disc* discs, Ctl* ctl, int d, int sp, int buf, long long n,
+                              const int32_t* c, const void* const v[4], unsigned* bad_out, int grid, cudaStream_t st);
 cudaError_t launch_unpack_state(int fp64, const Disc* discs, const Ctl* ctl, int d, int sp, int buf, long long cap,
-                                int32_t* c, void* const v[4], int grid, cudaStream_t st);
+                                int32_t* c, void* const v[4], long long* n_out, int grid, cudaStream_t st);
+cudaError_t launch_gather(const Gather& g, void* out, int sms, cudaStream_t st);
 long long sort_tile_chunks(int chunk);
 cudaError_t launch_load_profile(int fp64, const Disc* discs, int n_disc, Ctl* ctl, int buf, unsigned long long seed,
                                 const void* warm, int grid_x, cudaStream_t st);
@@ -48,8 +49,6 @@ cudaError_t launch_diag(int fp64, const Disc* discs, int n_disc, const Ctl* ctl,
                         int max_N, int grid_x, cudaStream_t st);
 size_t diag_smem(int max_N, unsigned mask, int bins);  // bins: 0 unless the launch samples the EEDF
 cudaError_t launch_set_dense(const Disc* discs, int n_disc, Ctl* ctl, int buf, cudaStream_t st);
-cudaError_t launch_finish_upload(const Disc* discs, Ctl* ctl, int d, int sp, long long n, const unsigned* bad,
-                                 int buf, cudaStream_t st);
 cudaError_t launch_debug_wait(int arrive, int tries, int* out, cudaStream_t st);
 cudaError_t launch_debug_philox(long long n, const uint32_t* ctr, uint32_t k0, uint32_t k1, uint32_t* out,
                                 cudaStream_t st);
