@@ -136,8 +136,11 @@ __device__ __forceinline__ unsigned long long cic_F(double f) {
 //   0 particles n_c; 1, 2 the sum of F = rn(f 2^32) as low and high 16-bit parts; node j then receives
 //     2^32 n_j - F_j + F_{j-1} (the charge split (2^32 - F, F) of every particle);
 //   3, 4 (electrons) the sums of the low 17 bits of the energy E and of its share H = rn(E f); node j
-//     receives E_j - H_j + H_{j-1}. The bits above (an electron of more than 32 eV) go straight to the
-//     global sums.
+//     receives E_j - H_j + H_{j-1}. The bits above (an electron of more than 32 eV) go to one more array, of
+//     one word per node (below 2^25), where shared memory holds it beside the rest (one electron in five is
+//     above 32 eV while the sheaths of a he_family discharge form, one in thirty later: global adds took
+//     26.1 us a step then, the array takes 24.4; 64 such discharges 84.2 -> 82.8), else straight to the
+//     global sums (above about 1970 cells of FP32: the array would cost a warp, 4 % of the sweep).
 // The 64-bit node values are formed when the CTA flushes. A piece sum stays below 2^32 while the CTA has
 // added at most FLUSH_PARTICLES particles of a species (plus as many newborns) since its last flush.
 template <typename T>
@@ -194,8 +197,8 @@ __device__ __forceinline__ void warp_dep(const Hist& h, int key, unsigned long l
 // Energy moment of the lanes' electrons (`on`; every lane of the warp calls) of energy speed^2 kappa_E
 // (2^-12 eV, clamped at 2^26) at (c, f).
 template <typename T>
-__device__ __forceinline__ void energy_add(const Hist& h, unsigned long long* Qg, bool on, int c, T f, T e2, T kappa_E,
-                                           int lane) {
+__device__ __forceinline__ void energy_add(const Hist& h, unsigned* hi, unsigned long long* Qg, bool on, int c, T f,
+                                           T e2, T kappa_E, int lane) {
     T eq = mul_(e2, kappa_E);
     if (!(eq <= (T)0x1p26)) eq = (T)0x1p26;
     const unsigned Et = rint_u32(eq), Eh = rint_u32(mul_(eq, f));
@@ -208,9 +211,14 @@ __device__ __forceinline__ void energy_add(const Hist& h, unsigned long long* Qg
     const bool high = on && (Et >> 17);
     if (__any_sync(FULL, high)) {
         if (high) {
-            const unsigned long long ht = Et >> 17, hh = Eh >> 17;
-            atomicAdd(&Qg[c], (ht - hh) << 17);
-            if (hh) atomicAdd(&Qg[c + 1], hh << 17);
+            const unsigned ht = Et >> 17, hh = Eh >> 17;
+            if (hi) {
+                if (ht != hh) atomicAdd(hi + c, ht - hh);
+                if (hh) atomicAdd(hi + c + 1, hh);
+            } else {
+                atomicAdd(&Qg[c], (unsigned long long)(ht - hh) << 17);
+                if (hh) atomicAdd(&Qg[c + 1], (unsigned long long)hh << 17);
+            }
         }
         __syncwarp();  // keeps this a branch: as predicated instructions the rare part costs every row 17 of them
     }
@@ -613,6 +621,8 @@ __host__ __device__ constexpr unsigned sweep_smem(int max_N, int sets, int warps
            (unsigned)sizeof(StoreSnap) * 2 * n_disc + 4u * 2 * (n_disc + 1);
 }
 
+constexpr unsigned SWEEP_SMEM_LIMIT = 227 * 1024 - 4096;  // dynamic shared memory; the static part is below 4 KB
+
 // Threads of a sweep CTA at most (one CTA per SM): the FP32 chunk code takes 80 registers (24 warps), the
 // FP64 code 128 (16 warps).
 template <typename T>
@@ -643,7 +653,7 @@ __host__ __device__ constexpr int sweep_max_threads() { return sizeof(T) == 4 ? 
 template <typename T, int PPT>
 __global__ void __launch_bounds__(sweep_max_threads<T>(), 1)
     k_sweep(const Disc* __restrict__ discs, int n_disc, Ctl* __restrict__ ctl, int in_buf, unsigned long long seed,
-            int max_N, int sets) {
+            int max_N, int sets, unsigned hi) {
     using R = typename Rec<T>::type;
     using T2 = typename T4<T>::two;
     constexpr int CHUNK = 32 * PPT;
@@ -661,6 +671,8 @@ __global__ void __launch_bounds__(sweep_max_threads<T>(), 1)
     uint8_t* Q = s_queue + warp * CHUNK;  // the chunk indices of the candidates, in slot order (CHUNK <= 256)
     StoreSnap* s_store = reinterpret_cast<StoreSnap*>(s_queue + NW * CHUNK);
     int* s_pre = reinterpret_cast<int*>(s_store + 2 * n_disc);  // [species][n_disc + 1]
+    // [node], behind everything else (0: none)
+    unsigned* const s_hi = hi ? reinterpret_cast<unsigned*>(smem_raw + hi) : nullptr;
 
     __shared__ Seg<T> s_seg[2];
     __shared__ long long s_step;
@@ -687,6 +699,7 @@ __global__ void __launch_bounds__(sweep_max_threads<T>(), 1)
     if (tid < NCNT) s_cnt[tid] = 0;
     load_seg(0);  // of a context with one discharge: nothing more to fetch after the wait
     for (int j = tid; j < sweep_hist_words(sets) * (max_N + WWORDS); j += nthr) s_win[j] = 0;
+    for (int j = tid; hi && j <= max_N; j += nthr) s_hi[j] = 0;
     __syncthreads();
     grid_dep_sync();
     auto load_field = [&]() {
@@ -896,7 +909,7 @@ __global__ void __launch_bounds__(sweep_max_threads<T>(), 1)
                 const T ef = fma_(rec.x, e.y, e.x);
                 const T vzn = fma_(Ksp, ef, rec.w);  // v_n
                 if (SP == 0)
-                    energy_add<T>(h, S.Qg, cand, c, rec.x, fma_(rec.y, rec.y, fma_(rec.z, rec.z, mul_(vzn, vzn))),
+                    energy_add<T>(h, s_hi, S.Qg, cand, c, rec.x, fma_(rec.y, rec.y, fma_(rec.z, rec.z, mul_(vzn, vzn))),
                                   S.k.kappa_E, lane);
                 if (cand) {
                     Cand<T> v{ef, rec.y, rec.z, S.leapfrog ? fma_(Ksp, ef, vzn) : vzn};  // leapfrog: at v_{n+1/2}
@@ -947,7 +960,7 @@ __global__ void __launch_bounds__(sweep_max_threads<T>(), 1)
                 const T ef = fma_(r.x, e.y, e.x);
                 const T vzn = fma_(Ksp, ef, r.w);  // v_n
                 if (SP == 0)
-                    energy_add<T>(h, S.Qg, valid && !coll, c, r.x, fma_(r.y, r.y, fma_(r.z, r.z, mul_(vzn, vzn))), kE,
+                    energy_add<T>(h, s_hi, S.Qg, valid && !coll, c, r.x, fma_(r.y, r.y, fma_(r.z, r.z, mul_(vzn, vzn))), kE,
                                   lane);
                 const T vz = coll ? r.w : fma_(Ksp, ef, vzn);
                 int cn;
@@ -1029,6 +1042,7 @@ __global__ void __launch_bounds__(sweep_max_threads<T>(), 1)
                     v += (unsigned long long)h[j - 1 + max_N] + ((unsigned long long)h[j - 1 + 2 * max_N] << 16);
                     if (sp == 0) q += h[j - 1 + 4 * max_N];
                 }
+                if (sp == 0 && hi) q += (unsigned long long)s_hi[j] << 17;
                 if (v) atomicAdd(&Dg[j], v);
                 if (sp == 0 && q) atomicAdd(&s_seg[0].Qg[j], q);
             }
@@ -1038,6 +1052,7 @@ __global__ void __launch_bounds__(sweep_max_threads<T>(), 1)
     auto clear = [&]() {
         __syncthreads();
         for (int j = tid; j < sweep_hist_words(sets) * max_N; j += nthr) s_h[j] = 0;  // the windows: in the flush
+        for (int j = tid; hi && j <= max_N; j += nthr) s_hi[j] = 0;
         if (tid < NCNT) s_cnt[tid] = 0;
         __syncthreads();
     };
@@ -2411,12 +2426,15 @@ static cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
 
 template <typename T, int PPT>
 static cudaError_t launch_sweep_t(const SweepLaunch& L) {
-    const size_t smem = sweep_smem<T, PPT>(L.max_N, L.sets, L.warps, L.n_disc);
+    const unsigned rest = sweep_smem<T, PPT>(L.max_N, L.sets, L.warps, L.n_disc);
+    const unsigned with_hi = rest + 4u * (L.max_N + 1);  // the array of the energies above 32 eV behind it
+    const unsigned hi = with_hi <= SWEEP_SMEM_LIMIT ? rest : 0u;
+    const size_t smem = hi ? with_hi : rest;
     auto kern = k_sweep<T, PPT>;
     cudaError_t e = smem_attr(kern, smem);
     if (e != cudaSuccess) return e;
     e = launch_pdl(kern, dim3(L.grid), dim3(32 * L.warps), smem, L.stream, L.discs, L.n_disc, L.ctl, L.in_buf, L.seed,
-                   L.max_N, L.sets);
+                   L.max_N, L.sets, hi);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
@@ -2438,11 +2456,10 @@ cudaError_t launch_sweep(const SweepLaunch& L) {
 // a quarter of the warps (above about 2900 cells).
 template <typename T, int PPT>
 static void sweep_shape_t(int max_N, int n_disc, int want, long long chunks, int* warps, int* sets) {
-    constexpr unsigned LIMIT = 227 * 1024 - 4096;  // the static part is below 4 KB
     const int top = sweep_max_threads<T>() / 32;
     int fit[3] = {0, 0, 0};
     for (int s = 1; s <= 2; ++s)
-        for (int w = 1; w <= top && sweep_smem<T, PPT>(max_N, s, w, n_disc) <= LIMIT; ++w) fit[s] = w;
+        for (int w = 1; w <= top && sweep_smem<T, PPT>(max_N, s, w, n_disc) <= SWEEP_SMEM_LIMIT; ++w) fit[s] = w;
     *sets = 4 * fit[2] >= 3 * fit[1] ? 2 : 1;
     int w = fit[*sets];
     if (want > 0 && want < w) w = want;
