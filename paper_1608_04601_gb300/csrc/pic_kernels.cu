@@ -473,16 +473,25 @@ __device__ __forceinline__ bool emit_see(const Seg<T>& S, unsigned long long* Do
     return true;
 }
 
-// Moves one record within a buffer (newborn compaction, dst <= src; nothing to do if equal).
+// Newborn compaction of a round: every lane's record src (where `on`) to dst <= src of the same buffer. All
+// lanes of the warp call. One lane's destination may be another's source, so all of them load before any
+// stores.
 template <typename T>
-__device__ __forceinline__ void move_rec(int32_t* c, void* p, unsigned src, unsigned dst) {
-    if (src == dst) return;
+__device__ __forceinline__ void compact_recs(int32_t* c, void* p, bool on, unsigned src, unsigned dst) {
     using R = typename Rec<T>::type;
     R* pp = reinterpret_cast<R*>(p);
-    const int cv = c[src];
-    const R rv = pp[src];
-    c[dst] = cv;
-    pp[dst] = rv;
+    const bool move = on && src != dst;
+    int cv = 0;
+    R rv{};
+    if (move) {
+        cv = c[src];
+        rv = pp[src];
+    }
+    __syncwarp();
+    if (move) {
+        c[dst] = cv;
+        pp[dst] = rv;
+    }
 }
 
 // n mod m and n / m for step numbers (32-bit operations below 2^31, the slow 64-bit ones out of line).
@@ -926,8 +935,8 @@ __global__ void __launch_bounds__(sweep_max_threads<T>(), 1)
                 if (SP == 0) {  // the round's newborns, from the candidates' ranks to parent-slot order (dst <= src)
                     const unsigned m1 = __ballot_sync(FULL, (o & 2u) != 0), m2 = __ballot_sync(FULL, (o & 4u) != 0);
                     if (m1 | m2) {
-                        if (o & 2u) move_rec<T>(S.sc, S.sp_, obase + q, offS + __popc(m1 & lt));
-                        if (o & 4u) move_rec<T>(S.bc, S.bp, obase + q, offB + __popc(m2 & lt));
+                        compact_recs<T>(S.sc, S.sp_, (o & 2u) != 0, obase + q, offS + __popc(m1 & lt));
+                        compact_recs<T>(S.bc, S.bp, (o & 4u) != 0, obase + q, offB + __popc(m2 & lt));
                         offS += __popc(m1);
                         offB += __popc(m2);
                         __syncwarp();
