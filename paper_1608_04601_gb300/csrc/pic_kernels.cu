@@ -55,7 +55,10 @@ template <> __device__ __forceinline__ const Seg<double>* segs_of<double>(const 
 // Programmatic dependent launch (the kernels of a step, launched by launch_pdl): wait until the
 // previous kernel in the stream has completed and its writes are visible. Every such kernel calls this
 // before its first access to memory that kernels write (a no-op for a kernel launched without the
-// attribute); what needs no results (shared memory cleared, constants fetched) may come before. No kernel
+// attribute); what needs no results (shared memory cleared, constants fetched) may come before. Memory that
+// the kernel before may still be writing when this one starts is not read-only over its lifetime, so it is
+// never read through the non-coherent path (__ldg, or a plain load from a const __restrict__ pointer), but
+// with __ldcg or from unrestricted pointers. No kernel
 // triggers its dependents early: they launch as its CTAs exit (with early triggers in the sweep and k_post
 // the smallest runs gained 0.6 us of 26 a step and the larger ones lost 1-2 %).
 __device__ __forceinline__ void grid_dep_sync() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -253,6 +256,13 @@ __device__ __forceinline__ void load_rec<double>(const void* p, unsigned i, doub
     const double2* pp = reinterpret_cast<const double2*>(p) + 2 * i;
     const double2 a = __ldcs(pp), b = __ldcs(pp + 1);
     f = a.x; vx = a.y; vy = b.x; vz = b.y;
+}
+
+// A whole record, coherent (see grid_dep_sync).
+__device__ __forceinline__ float4 ldcg_rec(const float4* p) { return __ldcg(p); }
+__device__ __forceinline__ d4 ldcg_rec(const d4* p) {
+    const double2 a = __ldcg(reinterpret_cast<const double2*>(p)), b = __ldcg(reinterpret_cast<const double2*>(p) + 1);
+    return d4{a.x, a.y, b.x, b.y};
 }
 
 // The random draws, directions and normals of a collision out of line: they appear several times in
@@ -1773,8 +1783,8 @@ __device__ __forceinline__ ChunkDesc chunk_desc(const Lay& L, long long n, const
     ChunkDesc c;
     if (k < L.K) {
         c.src = k * chunk;
-        c.base = __ldg(st + k);
-        c.cnt = __ldg(st + k + 1) - c.base;
+        c.base = __ldcg(st + k);
+        c.cnt = __ldcg(st + k + 1) - c.base;
     } else {
         const long long j = k - L.K;
         c.src = L.D0 + j * chunk;
@@ -1840,8 +1850,8 @@ __device__ __forceinline__ T col4(const T4r& r, int j) {
 constexpr int DIAG_BLOCK = 256, DIAG_NW = DIAG_BLOCK / 32;
 
 template <typename T>
-__global__ void __launch_bounds__(DIAG_BLOCK) k_diag(const Disc* __restrict__ discs, const Ctl* __restrict__ ctl,
-                                                     int buf, DiagArgs A) {
+__global__ void __launch_bounds__(DIAG_BLOCK) k_diag(const Disc* __restrict__ discs, const Ctl* ctl, int buf,
+                                                     DiagArgs A) {
     grid_dep_sync();
     extern __shared__ __align__(16) unsigned long long s_dg[];  // [arrays of the mask][N + 1], EEDF [bins] u32
     using R = typename Rec<T>::type;
@@ -1878,8 +1888,8 @@ __global__ void __launch_bounds__(DIAG_BLOCK) k_diag(const Disc* __restrict__ di
     const long long n = ctl->count[d][0];
     const Lay L = ctl->lay[d][0][buf];
     const long long chunks = chunks_of(L, n, CHUNK);
-    const int32_t* __restrict__ cc = D.c[buf][0];
-    const R* __restrict__ P = reinterpret_cast<const R*>(D.p[buf][0]);
+    const int32_t* cc = D.c[buf][0];
+    const R* P = reinterpret_cast<const R*>(D.p[buf][0]);
     for (long long k = (long long)blockIdx.x * DIAG_NW + warp; k < chunks; k += (long long)gridDim.x * DIAG_NW) {
         const ChunkDesc cd = chunk_desc(L, n, D.start[0], k, CHUNK);
         for (int r = 0; r < RPC; ++r) {
@@ -1887,8 +1897,8 @@ __global__ void __launch_bounds__(DIAG_BLOCK) k_diag(const Disc* __restrict__ di
             int c = -1;
             T f = 0, vx = 0, vy = 0, vz = 0;
             if (i < cd.cnt) {
-                c = cc[cd.src + i];
-                const R q = P[cd.src + i];
+                c = __ldcg(cc + cd.src + i);
+                const R q = ldcg_rec(P + cd.src + i);
                 f = q.x;
                 vx = q.y;
                 vy = q.z;
@@ -2105,11 +2115,9 @@ __global__ void __launch_bounds__(1024) k_sort_rows(const Disc* __restrict__ dis
 
 template <typename T>
 __global__ void __launch_bounds__(SORT_BLOCK) k_sort_scatter(const Disc* __restrict__ discs, int n_disc,
-                                                             const Ctl* __restrict__ ctl, int src, int dst,
-                                                             const unsigned* __restrict__ hist,
-                                                             const long long* __restrict__ hoff,
-                                                             const unsigned* __restrict__ tot,
-                                                             const unsigned* __restrict__ kr_all,
+                                                             const Ctl* ctl, int src, int dst, const unsigned* hist,
+                                                             const long long* __restrict__ hoff, const unsigned* tot,
+                                                             const unsigned* kr_all,
                                                              const long long* __restrict__ eoff) {
     __shared__ int s_pre[2 * MAXD + 1];
     grid_dep_sync();
@@ -2129,9 +2137,9 @@ __global__ void __launch_bounds__(SORT_BLOCK) k_sort_scatter(const Disc* __restr
         const R* __restrict__ ps = reinterpret_cast<const R*>(D.p[src][sp]);
         R* __restrict__ pd = reinterpret_cast<R*>(D.p[dst][sp]);
         int32_t* __restrict__ cd = D.c[dst][sp];
-        const unsigned* __restrict__ H = hist + hoff[seg] + (size_t)t * N;
-        const unsigned* __restrict__ cstart = tot + (long long)seg * MAXN;
-        const unsigned* __restrict__ KR = kr_all + eoff[seg] + (size_t)t * SORT_TILE + warp * (32 * SORT_R) + lane;
+        const unsigned* H = hist + hoff[seg] + (size_t)t * N;
+        const unsigned* cstart = tot + (long long)seg * MAXN;
+        const unsigned* KR = kr_all + eoff[seg] + (size_t)t * SORT_TILE + warp * (32 * SORT_R) + lane;
         const ChunkDesc my = lane < CPW && k0 + lane < chunks ? chunk_desc(L, n, D.start[sp], k0 + lane, CHUNK)
                                                              : ChunkDesc{0, 0, 0};
 #pragma unroll 1
@@ -2150,7 +2158,7 @@ __global__ void __launch_bounds__(SORT_BLOCK) k_sort_scatter(const Disc* __restr
 #pragma unroll
             for (int q = 0; q < B; ++q) {
                 const unsigned k = kr[q] & 0xFFFFu;  // a corrupt cell index (reported by the sweep): dropped
-                o[q] = k < (unsigned)N ? cstart[k] + H[k] + (kr[q] >> 16) : 0xFFFFFFFFu;
+                o[q] = k < (unsigned)N ? __ldcg(cstart + k) + __ldcg(H + k) + (kr[q] >> 16) : 0xFFFFFFFFu;
             }
 #pragma unroll
             for (int q = 0; q < B; ++q)
@@ -2174,8 +2182,8 @@ __global__ void k_repack(const Disc* __restrict__ discs, Ctl* __restrict__ ctl, 
     const Lay L = ctl->lay[d][sp][src];
     const long long chunks = chunks_of(L, n, CHUNK);
     using R = typename Rec<T>::type;
-    const R* __restrict__ ps = reinterpret_cast<const R*>(D.p[src][sp]);
-    const int32_t* __restrict__ cs_ = D.c[src][sp];
+    const R* ps = reinterpret_cast<const R*>(D.p[src][sp]);
+    const int32_t* cs_ = D.c[src][sp];
     R* __restrict__ pd = reinterpret_cast<R*>(D.p[dst][sp]);
     int32_t* __restrict__ cd = D.c[dst][sp];
     const int lane = threadIdx.x & 31;
@@ -2185,7 +2193,7 @@ __global__ void k_repack(const Disc* __restrict__ discs, Ctl* __restrict__ ctl, 
         const ChunkDesc c = chunk_desc(L, n, D.start[sp], k, CHUNK);
         for (int i = lane; i < c.cnt; i += 32) {
             cd[c.base + i] = __ldcs(cs_ + c.src + i);
-            pd[c.base + i] = ps[c.src + i];
+            pd[c.base + i] = ldcg_rec(ps + c.src + i);
         }
     }
 }
