@@ -353,7 +353,9 @@ pic_status pic_sweep_timing(pic_ctx* ctx, int32_t enable, double* total_ms, int6
 /* The bounded device-side wait of the sweep's bulk-copy staging, on its own: one mbarrier that
  * expects one arrival, polled at most `tries` times (1 .. 2^20). arrive = 0: nothing arrives, the
  * wait gives up and the call returns PIC_ERR_TIMEOUT with the device context intact (nothing is
- * left in flight); arrive = 1: PIC_OK. Synchronous, default stream.                        */
+ * left in flight); arrive = 1: PIC_OK; arrive = 2: one arrival, but one lane of the waiting warp
+ * gives up at once, and PIC_ERR_TIMEOUT again, as the warp answers as one. Synchronous, default
+ * stream.                                                                                  */
 pic_status pic_debug_wait(int32_t arrive, int32_t tries);
 pic_status pic_debug_philox(int64_t n, const uint32_t* ctr, const uint32_t key[2], uint32_t* out);
 /* Own log, sin(pi y), cos(pi y), Box-Muller and isotropic direction as used

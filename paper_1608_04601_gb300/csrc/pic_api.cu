@@ -1499,7 +1499,7 @@ extern "C" pic_status pic_debug_wait(int32_t arrive, int32_t tries) {
     if (cudaMalloc(&d, sizeof(int)) != cudaSuccess) return PIC_ERR_CUDA;
     int h = -1;
     cudaError_t e = cudaMemset(d, 0xFF, sizeof(int));
-    if (e == cudaSuccess) e = launch_debug_wait(arrive ? 1 : 0, tries, d, 0);
+    if (e == cudaSuccess) e = launch_debug_wait(arrive == 2 ? 2 : arrive ? 1 : 0, tries, d, 0);
     if (e == cudaSuccess) e = cudaMemcpy(&h, d, sizeof(int), cudaMemcpyDeviceToHost);
     cudaFree(d);
     if (e != cudaSuccess) return PIC_ERR_CUDA;

@@ -611,6 +611,11 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* mb, unsigned parit
     }
     return false;
 }
+// The same by a whole warp, with one answer for all its lanes: true only if none gave up (what follows is full
+// of warp-wide operations, so no lane may take another way than the rest).
+__device__ __forceinline__ bool warp_wait(unsigned long long* mb, unsigned parity, int tries = MBAR_TRIES) {
+    return __all_sync(FULL, mbar_wait(mb, parity, tries));
+}
 
 // Dynamic shared memory of the sweep: per cell the field and its difference to the next node (E_c,
 // E_{c+1} - E_c), the histograms (`sets` 2: both species at once, 5 + 3 arrays; 1: one species at a
@@ -1121,19 +1126,24 @@ __global__ void __launch_bounds__(sweep_max_threads<T>(), 1)
             if (pf_s != s) continue;
             const unsigned cs = (unsigned)pf_k;
             const int base = pf_base, cnt = pf_stop - pf_base, b = pf_b;
-            if (!mbar_wait(&s_mbar[warp][b], (phases >> b) & 1u)) err |= ERR_TIMEOUT;
+            if (!warp_wait(&s_mbar[warp][b], (phases >> b) & 1u)) {  // given up: the warp takes no more chunks
+                err |= ERR_TIMEOUT;
+                pf_s = n_store;
+                continue;
+            }
             phases ^= 1u << b;
             __syncwarp();
             prefetch_next();  // the warp's next chunk, into the other buffer
-            if (!(err & ERR_TIMEOUT)) {
-                unsigned char* buf = stage + (unsigned)b * sweep_stage_bytes<T, PPT>();
-                R* srec = reinterpret_cast<R*>(buf);
-                int32_t* scell = reinterpret_cast<int32_t*>(buf + REC_BYTES);
-                if (sp == 0) chunk(cs, base, cnt, srec, scell, IC<0>{}); else chunk(cs, base, cnt, srec, scell, IC<1>{});
-            }
+            unsigned char* buf = stage + (unsigned)b * sweep_stage_bytes<T, PPT>();
+            R* srec = reinterpret_cast<R*>(buf);
+            int32_t* scell = reinterpret_cast<int32_t*>(buf + REC_BYTES);
+            if (sp == 0) chunk(cs, base, cnt, srec, scell, IC<0>{}); else chunk(cs, base, cnt, srec, scell, IC<1>{});
             __syncwarp();
         }
     }
+    // a copy is in flight past this point only if its wait was given up (each one issued is of a chunk this warp
+    // takes, and the next is issued after the wait): the one of buffer pf_b, waited for once more, with a limit
+    if (err & ERR_TIMEOUT) mbar_wait(&s_mbar[warp][pf_b], (phases >> pf_b) & 1u);
     if (cur_d >= 0) flush(cur_sp);
     if (err) atomicOr(&s_err, err);
     __syncthreads();
@@ -2387,18 +2397,21 @@ __global__ void k_debug_math(long long n, const float* __restrict__ x, const flo
 
 namespace pic {
 
-// Bounded-wait check: one mbarrier expecting a single arrival. With arrive = 0 nothing arrives, so
+// Bounded-wait check, one warp: one mbarrier expecting a single arrival. With arrive = 0 nothing arrives, so
 // the wait gives up after `tries` polls and the kernel reports ERR_TIMEOUT in *out; nothing is in
-// flight when it returns. With arrive = 1 the thread arrives first and the wait succeeds.
+// flight when it returns. With arrive = 1 a thread arrives first and the wait succeeds. With arrive = 2 a
+// thread arrives but lane 0 gives up without a poll: every lane has to report the timeout (ERR_NONFINITE if
+// they differ).
 __global__ void k_debug_wait(int arrive, int tries, int* out) {
     __shared__ __align__(8) unsigned long long mb;
     if (threadIdx.x == 0) mbar_init(&mb);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncthreads();
-    if (threadIdx.x == 0) {
-        if (arrive) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&mb)) : "memory");
-        *out = mbar_wait(&mb, 0u, tries) ? 0 : ERR_TIMEOUT;
-    }
+    if (threadIdx.x == 0 && arrive)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&mb)) : "memory");
+    const bool got = warp_wait(&mb, 0u, arrive == 2 && threadIdx.x == 0 ? 0 : tries);
+    const unsigned m = __ballot_sync(FULL, got);
+    if (threadIdx.x == 0) *out = m == FULL ? 0 : m == 0 ? ERR_TIMEOUT : ERR_NONFINITE;
 }
 
 // Raises a kernel's dynamic shared-memory limit once per (kernel, size). Kernels

@@ -315,9 +315,9 @@ class Simulation:
         return ms.value, n.value
 
 
-def debug_wait(arrive: bool, tries: int) -> int:
+def debug_wait(arrive: int, tries: int) -> int:
     """Status of pic_debug_wait (PIC_OK or PIC_ERR_TIMEOUT), returned rather than raised."""
-    return int(NV.lib().pic_debug_wait(1 if arrive else 0, int(tries)))
+    return int(NV.lib().pic_debug_wait(int(arrive), int(tries)))
 
 
 def debug_philox(ctr: np.ndarray, key) -> np.ndarray:
