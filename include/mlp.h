@@ -49,7 +49,8 @@ int64_t mlp_param_count(const mlp_ctx* ctx);
 pic_status mlp_set_params(mlp_ctx* ctx, const float* host);
 pic_status mlp_get_params(mlp_ctx* ctx, float* host);
 
-/* y[batch x sizes[n_layers]] = network(x[batch x sizes[0]]); batch <= max_batch. */
+/* y[batch x sizes[n_layers]] = network(x[batch x sizes[0]]); batch <= max_batch;
+ * x and y may overlap.                                                      */
 pic_status mlp_forward(mlp_ctx* ctx, int32_t batch, const float* x, float* y);
 
 /* Forward and backward of L = mean over batch x outputs of (y - t)^2: *loss

@@ -768,7 +768,14 @@ pic_status mlp_get_params(mlp_ctx* c, float* host) {
 
 pic_status mlp_forward(mlp_ctx* c, int32_t batch, const float* x, float* y) {
     if (!c || !x || !y || batch < 1 || batch > c->max_batch) return PIC_ERR_ARG;
-    const cudaError_t e = forward(c, batch, x, y, nullptr, nullptr);
+    // With one layer the only product reads x in every column tile and writes y as tiles finish: if the two
+    // overlap, the outputs go through the context's own array. (With more layers x is read by the first
+    // launch and y written by the last.)
+    const size_t nx = sizeof(float) * (size_t)batch * c->sizes[0], ny = sizeof(float) * (size_t)batch * c->sizes[c->L];
+    const uintptr_t ax = reinterpret_cast<uintptr_t>(x), ay = reinterpret_cast<uintptr_t>(y);
+    const bool own = c->L == 1 && ax < ay + ny && ay < ax + nx;
+    cudaError_t e = forward(c, batch, x, own ? c->y32[0] : y, nullptr, nullptr);
+    if (e == cudaSuccess && own) e = cudaMemcpyAsync(y, c->y32[0], ny, cudaMemcpyDeviceToDevice, c->stream);
     return e == cudaSuccess ? PIC_OK : fail(c, PIC_ERR_CUDA, "forward", e);
 }
 
