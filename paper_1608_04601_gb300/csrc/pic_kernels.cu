@@ -2390,10 +2390,8 @@ __global__ void k_debug_math(long long n, const float* __restrict__ x, const flo
 
 // ---------------------------------------------------------------------------
 // Launch wrappers used by the host runtime.
-#include <mutex>
-#include <vector>
-
 #include "pic_launch.h"
+#include "pic_limits.h"
 
 namespace pic {
 
@@ -2414,24 +2412,9 @@ __global__ void k_debug_wait(int arrive, int tries, int* out) {
     if (threadIdx.x == 0) *out = m == FULL ? 0 : m == 0 ? ERR_TIMEOUT : ERR_NONFINITE;
 }
 
-// Raises a kernel's dynamic shared-memory limit once per (kernel, size). Kernels
-// are told apart by their address (instantiations can share a type).
 template <typename K>
 static cudaError_t smem_attr(K kern, size_t smem) {
-    static std::mutex mu;
-    static std::vector<std::pair<const void*, size_t>> done;
-    std::lock_guard<std::mutex> lk(mu);
-    const void* key = reinterpret_cast<const void*>(kern);
-    for (auto& p : done)
-        if (p.first == key) {
-            if (smem <= p.second) return cudaSuccess;
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e == cudaSuccess) p.second = smem;
-            return e;
-        }
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) done.push_back({key, smem});
-    return e;
+    return raise_smem_limit(reinterpret_cast<const void*>(kern), smem);
 }
 
 // Launch with programmatic stream serialization: the grid may be scheduled while the kernel before
@@ -2513,15 +2496,12 @@ cudaError_t launch_finalize(int fp64, const Disc* discs, int n_disc, Ctl* ctl, i
     const int nsl = (mode & 1) ? (max_slices > 0 ? max_slices : 1) : 0;
     const int parts = (mode & 8) ? 1 : max_N / FIELD_NODES + 2;  // field parts (y even), totals and moments parts (odd)
     const dim3 grid(nsl + parts, 2 * n_disc);
-    if (fp64) {
-        smem_attr(k_post<double>, smem);
+    const cudaError_t e = fp64 ? smem_attr(k_post<double>, smem) : smem_attr(k_post<float>, smem);
+    if (e != cudaSuccess) return e;
+    if (fp64)
         return launch_pdl(k_post<double>, grid, dim3(POST_BLOCK), smem, st, discs, n_disc, ctl, out_buf, mode, nsl,
                           max_N);
-    } else {
-        smem_attr(k_post<float>, smem);
-        return launch_pdl(k_post<float>, grid, dim3(POST_BLOCK), smem, st, discs, n_disc, ctl, out_buf, mode, nsl,
-                          max_N);
-    }
+    return launch_pdl(k_post<float>, grid, dim3(POST_BLOCK), smem, st, discs, n_disc, ctl, out_buf, mode, nsl, max_N);
 }
 
 cudaError_t launch_load(int fp64, const Disc* discs, int n_disc, Ctl* ctl, int buf, unsigned long long seed,
