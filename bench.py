@@ -366,7 +366,7 @@ def run_gpu(args, rank: int, world: int):
     if args.autotune:
         # small search of the launch shape and the sort period on this workload (whole steps, L2 flushed)
         from paper_1608_04601_gb300 import autotune
-        tuned = autotune.autotune([gas], [(d, 0)], "fp32", tiles=[(256, 2), (256, 4), (128, 4)], ctas=[0],
+        tuned = autotune.autotune([gas], [(d, 0)], "fp32", tiles=[(256, 2), (256, 4)], ctas=[0],
                                   sorts=[8, 16], use_cache=False)
         args.block, args.ppt, args.sort_every = tuned["block"], tuned["ppt"], tuned["sort_every"]
     sort_every = args.sort_every

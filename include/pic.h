@@ -106,9 +106,10 @@ typedef struct {
                              /* after every step n with (n+1) % K == 0       */
     int32_t block;           /* 128, 256 (default), 512: see ctas_per_sm     */
     int32_t ppt;             /* sweep particles per thread: 2, 4 (default), 8 */
-    int32_t ctas_per_sm;     /* sweep threads per SM at most, in units of    */
-                             /* block (0: as many as fit); the sweep runs one */
-                             /* CTA of them per SM                           */
+                             /* (8 with block 512 counts as 4)               */
+    int32_t ctas_per_sm;     /* limit on the sweep's threads per SM, in      */
+                             /* units of block (0: as many as fit, whatever  */
+                             /* block is); the sweep runs one CTA per SM     */
     int32_t use_graph;       /* 1: replay pic_step in CUDA graphs of one rf  */
                              /* period (requires sort_every | steps/period)  */
     void* cuda_stream;       /* cudaStream_t to enqueue on; NULL = own stream */

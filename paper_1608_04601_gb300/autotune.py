@@ -1,10 +1,11 @@
 """Autotuner of the sweep's launch shape and the sort period.
 
-Searches the sweep tile (threads per CTA x particles per thread), persistent CTAs per SM and
-the stable-sort period K over a small grid, timing whole steps with CUDA events (L2 flushed
-before each timed step, as in the benchmark), and caches the fastest choice per (workload,
-precision, GPU) in a JSON file next to this module. The search itself only calls the library's
-public API.
+The sweep runs one CTA per SM. Searched are the particles per thread (the chunk of a warp), the
+limit on the CTA's threads (block x ctas_per_sm; ctas_per_sm = 0: as many as fit, whatever block
+is) and the stable-sort period K, over a small grid, timing whole steps with CUDA events (L2 flushed
+before each timed step, as in the benchmark). Candidates that are the same launch are timed once.
+The fastest choice per (workload, precision, GPU) is cached in a JSON file next to this module. The
+search itself only calls the library's public API.
 """
 from __future__ import annotations
 
@@ -16,8 +17,23 @@ from . import pic
 
 CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_autotune_cache.json")
 
-TILES = [(256, 4), (256, 2), (128, 4), (256, 8), (128, 8)]
-CTAS = [0, 1]
+TILES = [(128, 4), (128, 2), (128, 8)]  # block, particles per thread
+CTAS = [0, 5, 2]  # with blocks of 128: as many threads as fit, at most 640, at most 256
+MAX_THREADS = {"fp32": 768, "fp64": 512}  # of a sweep CTA
+
+
+def launch_shapes(tiles, ctas, precision: str) -> list:
+    """The (block, ppt, ctas_per_sm) candidates of the grid that differ in the sweep's launch: its chunk
+    and its limit on threads."""
+    out, seen = [], set()
+    top = MAX_THREADS[precision]
+    for block, ppt in tiles:
+        for c in ctas:
+            shape = (4 if block == 512 and ppt == 8 else ppt, min(top, block * c) if c else top)
+            if shape not in seen:
+                seen.add(shape)
+                out.append((block, ppt, c))
+    return out
 
 
 def sort_periods(steps_per_period: int, choices=(1, 2, 4, 8, 16, 32, 64)) -> list:
@@ -82,17 +98,16 @@ def autotune(gases, discharges, precision: str = "fp32", tiles=None, ctas=None, 
     spp = discharges[0][0].steps_per_period
     best = None
     results = []
-    for block, ppt in (tiles or TILES):
-        for c in (ctas or CTAS):
-            for k in (sorts or sort_periods(spp)):
-                # warm-up through the first sort, then two whole sort periods
-                ms = time_config(gases, discharges, precision, block, ppt, c, k, steps=max(12, 2 * k),
-                                 warmup=max(4, k))
-                results.append({"block": block, "ppt": ppt, "ctas_per_sm": c, "sort_every": k, "ms_per_step": ms})
-                if log:
-                    log(results[-1])
-                if best is None or ms < best["ms_per_step"]:
-                    best = results[-1]
+    for block, ppt, c in launch_shapes(tiles or TILES, ctas or CTAS, precision):
+        for k in (sorts or sort_periods(spp)):
+            # warm-up through the first sort, then two whole sort periods
+            ms = time_config(gases, discharges, precision, block, ppt, c, k, steps=max(12, 2 * k),
+                             warmup=max(4, k))
+            results.append({"block": block, "ppt": ppt, "ctas_per_sm": c, "sort_every": k, "ms_per_step": ms})
+            if log:
+                log(results[-1])
+            if best is None or ms < best["ms_per_step"]:
+                best = results[-1]
     best = dict(best)
     best["searched"] = len(results)
     cache[key] = best
