@@ -717,8 +717,11 @@ pic_status mlp_create(mlp_ctx** out, int32_t n_layers, const int32_t* sizes, int
               dalloc(c, &c->mse_part, (size_t)((max_batch + TBM - 1) / TBM) * ((wmax + 15) / 16)) &&
               cudaHostAlloc(&c->h_err, sizeof(unsigned), cudaHostAllocMapped) == cudaSuccess &&
               cudaHostGetDevicePointer(&c->d_err, c->h_err, 0) == cudaSuccess;
-    for (int l = 0; l < n_layers && ok; ++l)
-        ok = dalloc(c, &c->y32[l], (size_t)max_batch * sizes[l + 1]) && dalloc(c, &c->y16[l], (size_t)pad16(max_batch) * c->ld[l + 1]);
+    // hidden layers' outputs (the last layer writes y or the error; of a single layer, y may go through y32[0])
+    for (int l = 0; l < n_layers && ok; ++l) {
+        if (l + 1 < n_layers) ok = dalloc(c, &c->y16[l], (size_t)pad16(max_batch) * c->ld[l + 1]);
+        if (l + 1 < n_layers || n_layers == 1) ok = ok && dalloc(c, &c->y32[l], (size_t)max_batch * sizes[l + 1]);
+    }
     for (int b = 0; b < 2 && ok; ++b)
         ok = dalloc(c, &c->g32[b], (size_t)max_batch * wmax) && dalloc(c, &c->g16[b], (size_t)pad16(max_batch) * wmax);
     if (!ok) {

@@ -395,7 +395,6 @@ extern "C" pic_status pic_batch_create(pic_ctx** out, const pic_gas* gases, int3
         ctx->gas.push_back(gd);
     }
 
-    const long long tile = (long long)o.block * o.ppt;
     const long long chunk = 32ll * o.ppt;
     auto bcap_of = [&](int i) {
         return std::max(ctx->dis[i].weights.capacity_e, ctx->dis[i].weights.capacity_i) / 8 + 4096;
@@ -514,9 +513,7 @@ extern "C" pic_status pic_batch_create(pic_ctx** out, const pic_gas* gases, int3
         ALLOC(D.V_hist, double*, sizeof(double) * PERIOD_HIST);
         D.has_see = d.weights.gamma_see > 0.0;
         D.leapfrog = o.leapfrog != 0;
-        D.tile = (int)tile;
         D.chunk = 32 * o.ppt;
-        D.warps = o.block / 32;
         D.rec_words = ctx->fp64 ? 2 : 1;
         fill_consts<float>(D.cf, der, d);
         fill_consts<double>(D.cd, der, d);

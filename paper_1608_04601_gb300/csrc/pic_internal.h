@@ -99,9 +99,9 @@ struct Disc {
     // rho = pc_w[1] D_i - pc_w[0] D_e (half-cell volume); 1/dx, -1/(2 dx), dx/(2 eps0), 1/N
     double pc_r[2], pc_w[2], inv_dx, m_inv_2dx, hdx_eps, inv_N, inv_dt;
     const double* V0tab;      // V_rf sin(2 pi f k dt), k < steps_per_period, or null (then sin on device)
-    int has_see, tile;        // sweep tile (slots) of this context
-    int leapfrog, pad_lf;     // push scheme: 0 velocity Verlet (collisions at v_n), 1 leapfrog (at v_{n+1/2})
-    int chunk, warps;         // compaction unit: one warp's 32 PPT slots; warps per tile
+    int has_see;
+    int leapfrog;             // push scheme: 0 velocity Verlet (collisions at v_n), 1 leapfrog (at v_{n+1/2})
+    int chunk;                // compaction unit: one warp's 32 PPT slots
     int rec_words;            // particle record size in 16-byte words (1: FP32, 2: FP64)
     Consts<float> cf;
     Consts<double> cd;
@@ -180,8 +180,6 @@ struct DiagArgs {
 // Control block; one per context, in device memory.
 struct Ctl {
     long long step;           // current step index n
-    unsigned int tile_ctr;    // sweep tile dispenser
-    unsigned int done;        // sweep CTAs finished
     unsigned int fin_done;    // k_post CTAs finished
     int error;                // ERR_* bits
     long long count[MAXD][2]; // superparticles per store
