@@ -56,7 +56,7 @@ enum Epilogue {
 struct GemmArgs {
     const bf16* A;
     const bf16* B;
-    const float* A32;    // FP32 source of A (M rows of K, K-major), converted while staged and kept in A16
+    const float* A32;    // FP32 source of A (M rows of K <= TBK, K-major), converted while staged, kept in A16
     bf16* A16;
     int lda, ldb, a_t, b_t;
     int M, N, K;
@@ -149,23 +149,44 @@ __device__ __forceinline__ unsigned fetch(uint32_t s, const bf16* X, int ld, int
     return copies * bytes;
 }
 
-// A chunk of A from FP32 (K-major), converted by all threads; the first CTA of a row of tiles keeps the
-// converted operand (for the weight gradients), with its padding.
-__device__ __forceinline__ void stage_f32(unsigned char* s, const GemmArgs& g, int m0, int k0, int kcs, bool keep) {
+// 8 BF16 of row r from column k of an FP32 array of M rows of K (zeros outside).
+__device__ __forceinline__ uint4 bf16_group(const float* x, int M, int K, int r, int k) {
+    uint32_t w[4] = {0u, 0u, 0u, 0u};
+    if (r < M) {
+        x += (size_t)r * K + k;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (k + i < K) w[i >> 1] |= (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(x[i])) << (16 * (i & 1));
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// A from FP32 (K-major, one chunk of kcs groups of 8 k), converted by all threads; the first CTA of a row of
+// tiles keeps the converted operand (for the weight gradients), with its padding.
+__device__ __forceinline__ void stage_f32(unsigned char* s, const GemmArgs& g, int m0, int kcs, bool keep) {
     const int rows = min(TBM, pad16(g.M) - m0);
 #pragma unroll 1
     for (int u = threadIdx.x; u < rows * kcs; u += TTHREADS) {
-        const int r = u / kcs, kc = u % kcs, k = k0 + 8 * kc;
-        uint32_t w[4] = {0u, 0u, 0u, 0u};
-        if (m0 + r < g.M) {
-            const float* x = g.A32 + (size_t)(m0 + r) * g.K + k;
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-                if (k + i < g.K) w[i >> 1] |= (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(__ldcg(x + i))) << (16 * (i & 1));
-        }
-        const uint4 v = make_uint4(w[0], w[1], w[2], w[3]);
-        if (keep) *reinterpret_cast<uint4*>(g.A16 + cm_index(m0 + r, k, g.lda)) = v;
+        const int r = u / kcs, kc = u % kcs;
+        const uint4 v = bf16_group(g.A32, g.M, g.K, m0 + r, 8 * kc);
+        if (keep) *reinterpret_cast<uint4*>(g.A16 + cm_index(m0 + r, 8 * kc, g.lda)) = v;
         *reinterpret_cast<uint4*>(s + (r >> 3) * (TBK * 16) + kc * CM + (r & 7) * 16) = v;
+    }
+}
+
+// An input of more than one chunk: converted into core matrices once, by a launch of its own, and fetched
+// through the ring like every other operand. (Converted while staged in the product, a chunk had to wait for
+// the products of the chunk before, in every column tile again. A forward pass, that way -> this way: 784-512-10
+// at batch 4096 99 -> 37 us, at 256 56 -> 18, 4096-4096 at batch 4096 2595 -> 503, 129-64-10 at batch 16,
+// two chunks, 10.9 -> 9.2.) A warp takes 8 rows of 4 groups of 8 k: 128 contiguous bytes of each row in, 512
+// contiguous bytes out.
+__global__ void __launch_bounds__(256) k_input_bf16(const float* x, bf16* x16, int M, int K, int ld) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int lane = threadIdx.x & 31, groups = ld >> 3, quads = (groups + 3) >> 2;
+    const int items = pad16(M) / 8 * quads, step = gridDim.x * 8;
+    for (int i = blockIdx.x * 8 + (threadIdx.x >> 5); i < items; i += step) {
+        const int r = i / quads * 8 + (lane & 7), kc = i % quads * 4 + (lane >> 3);
+        if (kc < groups) *reinterpret_cast<uint4*>(x16 + cm_index(r, 8 * kc, ld)) = bf16_group(x, M, K, r, 8 * kc);
     }
 }
 
@@ -234,8 +255,7 @@ __global__ void __launch_bounds__(TTHREADS) k_gemm(const __grid_constant__ Launc
     const int tn = (g.N + TBN - 1) / TBN, m0 = tile / tn * TBM, n0 = tile % tn * TBN;
     const int Kp = pad16(g.K), nk = (Kp + TBK - 1) / TBK;
     asm volatile("griddepcontrol.wait;" ::: "memory");  // nothing above reads what kernels write
-    // FP32 input (the first layer): chunk 0 by all threads; a wider input takes the chunks one by one below
-    if (g.A32) stage_f32(smem, g, m0, 0, min(TBK, Kp) / 8, n0 == 0 && g.A16);
+    if (g.A32) stage_f32(smem, g, m0, Kp / 8, n0 == 0);  // FP32 input (of one chunk): by all threads
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -277,30 +297,7 @@ __global__ void __launch_bounds__(TTHREADS) k_gemm(const __grid_constant__ Launc
                      : "memory");
     };
     bool ok = true;
-    if (g.A32 && nk > 1) {  // one chunk at a time: staged by all threads, its products waited for
-        for (int i = 0; i < nk; ++i) {
-            if (i > 0) {
-                if (__syncthreads_or(!tc_wait(freed, (unsigned)(i - 1) & 1u))) {
-                    ok = false;
-                    break;
-                }
-                stage_f32(smem, g, m0, i * TBK, min(TBK, Kp - i * TBK) / 8, n0 == 0 && g.A16);
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                __syncthreads();
-            }
-            if (warp == 0) load(i, 0);
-            const bool here = tc_wait(landed, (unsigned)i & 1u);
-            if (__syncthreads_or(!here)) {
-                ok = false;
-                break;
-            }
-            if (tid == 0) {
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                products(i, 0);
-            }
-        }
-        if (!ok && tid == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(all_done) : "memory");
-    } else if (warp == 0) {  // the copies
+    if (warp == 0) {  // the copies
         int s = 0;
         unsigned phase = 1;
         for (int i = 0; i < nk; ++i) {
@@ -634,9 +631,14 @@ cudaError_t forward(mlp_ctx* c, int batch, const float* x, float* y, const float
         GemmArgs& g = L.g[0];
         g.A = l == 0 ? c->x16 : c->y16[l - 1];
         g.lda = c->ld[l];
-        if (l == 0) {
+        if (l == 0 && c->ld[0] <= TBK) {
             g.A32 = x;
             g.A16 = c->x16;
+        } else if (l == 0) {
+            const int items = pad16(batch) / 8 * ((c->ld[0] / 8 + 3) / 4);  // of a warp, eight warps a CTA
+            e = launch_pdl(c, k_input_bf16, dim3(std::min((items + 7) / 8, 8 * c->num_sms)), 256, 0, x, c->x16, batch, in,
+                           c->ld[0]);
+            if (e != cudaSuccess) break;
         }
         g.B = c->w16 + c->w16off[l];
         g.ldb = c->ld[l];
@@ -771,12 +773,12 @@ pic_status mlp_get_params(mlp_ctx* c, float* host) {
 
 pic_status mlp_forward(mlp_ctx* c, int32_t batch, const float* x, float* y) {
     if (!c || !x || !y || batch < 1 || batch > c->max_batch) return PIC_ERR_ARG;
-    // With one layer the only product reads x in every column tile and writes y as tiles finish: if the two
-    // overlap, the outputs go through the context's own array. (With more layers x is read by the first
-    // launch and y written by the last.)
+    // A single launch (one layer, its input within one chunk) reads x in every column tile and writes y as
+    // tiles finish: if the two overlap, the outputs go through the context's own array. (Otherwise x is read
+    // by the first launch and y written by the last.)
     const size_t nx = sizeof(float) * (size_t)batch * c->sizes[0], ny = sizeof(float) * (size_t)batch * c->sizes[c->L];
     const uintptr_t ax = reinterpret_cast<uintptr_t>(x), ay = reinterpret_cast<uintptr_t>(y);
-    const bool own = c->L == 1 && ax < ay + ny && ay < ax + nx;
+    const bool own = c->L == 1 && c->ld[0] <= TBK && ax < ay + ny && ay < ax + nx;
     cudaError_t e = forward(c, batch, x, own ? c->y32[0] : y, nullptr, nullptr);
     if (e == cudaSuccess && own) e = cudaMemcpyAsync(y, c->y32[0], ny, cudaMemcpyDeviceToDevice, c->stream);
     return e == cudaSuccess ? PIC_OK : fail(c, PIC_ERR_CUDA, "forward", e);
