@@ -2167,8 +2167,11 @@ __global__ void __launch_bounds__(SORT_BLOCK) k_sort_scatter(const Disc* __restr
             }
 #pragma unroll
             for (int q = 0; q < B; ++q) {
-                const unsigned k = kr[q] & 0xFFFFu;  // a corrupt cell index (reported by the sweep): dropped
-                o[q] = k < (unsigned)N ? __ldcg(cstart + k) + __ldcg(H + k) + (kr[q] >> 16) : 0xFFFFFFFFu;
+                // A corrupt cell index (reported by the sweep): dropped. Coherent loads by their unrestricted
+                // pointers, through L1: a tile's slots meet in one row of H. With __ldcg, which asks L2 for
+                // each slot: 1e6 + 1e6 in 64 cells 36 -> 47 us, unsorted in 512 cells 63 -> 117.
+                const unsigned k = kr[q] & 0xFFFFu;
+                o[q] = k < (unsigned)N ? cstart[k] + H[k] + (kr[q] >> 16) : 0xFFFFFFFFu;
             }
 #pragma unroll
             for (int q = 0; q < B; ++q)

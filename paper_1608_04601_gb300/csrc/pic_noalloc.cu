@@ -37,8 +37,10 @@ void* g_scratch_addr[256] = {};
 
 // Three kernels: tile counts, their scans (sort_rows), scatter. No scratch holds the ranks, so the scatter
 // forms them again from the cells. Each waits for the one before it. Bounded by latency at 1e6 particles: the
-// loads of a warp's eight rows go out together. 1e6 particles in 512 cells: 39 -> 26 us a call (before: four kernels,
-// one row's loads at a time, two passes over the cells in the scatter).
+// loads of a warp's eight rows go out together. 1e6 particles in 512 cells, nearly sorted: 37 -> 21 us a call, in
+// random order 55 -> 33 (before: four kernels, one row's loads at a time, two passes over the cells in the
+// scatter). The scatter reads a tile's offsets through L1 (plain loads of unrestricted pointers: the row scan
+// may still write them when this grid starts); asking L2 for each slot took 61 us in random order.
 __global__ void __launch_bounds__(SORT_BLOCK) na_count(const int32_t* __restrict__ c, long long n, int N,
                                                        unsigned* __restrict__ hist, long long Ts) {
     extern __shared__ unsigned s_c[];
@@ -116,7 +118,7 @@ __global__ void __launch_bounds__(SORT_BLOCK, 2) na_scatter(const int32_t* __res
 #pragma unroll
             for (int q = 0; q < B; ++q) {
                 const unsigned c = k[r0 + q] & 0xFFFFu;
-                o[q] = c < (unsigned)N ? __ldcg(cstart + c) + __ldcg(hist + t * N + c) + W[c] + (k[r0 + q] >> 16) : 0xFFFFFFFFu;
+                o[q] = c < (unsigned)N ? cstart[c] + hist[t * N + c] + W[c] + (k[r0 + q] >> 16) : 0xFFFFFFFFu;
                 if (r0 > 0 && b + 32 * (r0 + q) < n) rec[q] = ps[b + 32 * (r0 + q)];
             }
 #pragma unroll

@@ -22,12 +22,10 @@ __device__ __forceinline__ unsigned row_rank(unsigned short* W, unsigned k, unsi
         }
     } else {
         const unsigned peers = __match_any_sync(FULL, k);
-        if (k < N) {
-            const unsigned b = W[k];
-            rank = b + __popc(peers & lt);
-            __syncwarp(peers);
-            if (lane == __ffs(peers) - 1) W[k] = (unsigned short)(b + __popc(peers));
-        }
+        const unsigned b = k < N ? W[k] : 0u;
+        if (k < N) rank = b + __popc(peers & lt);
+        __syncwarp();  // of the whole warp: one per group of equal cells runs as many times as there are groups
+        if (k < N && lane == __ffs(peers) - 1) W[k] = (unsigned short)(b + __popc(peers));
     }
     __syncwarp();
     return rank;
