@@ -100,6 +100,7 @@ struct Disc {
     double pc_r[2], pc_w[2], inv_dx, m_inv_2dx, hdx_eps, inv_N, inv_dt;
     const double* V0tab;      // V_rf sin(2 pi f k dt), k < steps_per_period, or null (then sin on device)
     int has_see;
+    int jh;                   // entries of the ring J_hist
     int leapfrog;             // push scheme: 0 velocity Verlet (collisions at v_n), 1 leapfrog (at v_{n+1/2})
     int chunk;                // compaction unit: one warp's 32 PPT slots
     int rec_words;            // particle record size in 16-byte words (1: FP32, 2: FP64)
@@ -145,7 +146,6 @@ struct Disc {
     // discharge current density J(t) at z = 0 and z = d of every step, ring of jh steps, and the
     // first-harmonic amplitude of J at z = 0 of every rf period (ring of PERIOD_HIST)
     double* J_hist;           // [jh][2]
-    int jh;
     const double* jtab;       // sin, cos of 2 pi f (k + 1/2) dt, k < steps_per_period, or null
     double* J_amp;            // [PERIOD_HIST]
     double* V_hist;           // [PERIOD_HIST] rf voltage amplitude applied in every period
@@ -180,7 +180,6 @@ struct DiagArgs {
 // Control block; one per context, in device memory.
 struct Ctl {
     long long step;           // current step index n
-    unsigned int fin_done;    // k_post CTAs finished
     int error;                // ERR_* bits
     long long count[MAXD][2]; // superparticles per store
     Lay lay[MAXD][2][2];      // [discharge][species][buffer] layout of the store in that buffer
@@ -202,6 +201,7 @@ struct Ctl {
     double J_drive[MAXD];
     double period_acc[MAXD][2];   // sum of the counts over the steps of the current rf period
     unsigned sort_rows_done[MAXD][2];  // k_sort_rows CTAs finished, per store (reset by the last)
+    unsigned fin_done;        // k_post CTAs finished; apart from the words that its other CTAs still read
     unsigned up_bad, up_done;  // state upload: cells out of range, CTAs finished (both 0 between uploads)
 };
 
