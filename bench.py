@@ -82,7 +82,7 @@ def recorded_traffic(prec: str, kernel: str, workload_name: str):
     return e
 
 
-def sweep_roofline(r: dict, prec: str, block: int, ppt: int, workload_name: str) -> dict:
+def sweep_roofline(r: dict, prec: str, ppt: int, workload_name: str) -> dict:
     """Roofline of the dominant kernel (the sweep) from one measure() result: algorithmic bytes per
     launch (40 B per particle-step in FP32, 72 B in FP64, times the particles one launch processes)
     over the average CUDA-event duration of the sweep launches of the timed steps."""
@@ -91,7 +91,7 @@ def sweep_roofline(r: dict, prec: str, block: int, ppt: int, workload_name: str)
     bytes_per_launch = BYTES_PER_PS[prec] * launch_ps
     avg_sweep_s = r["sweep_ms"] * 1e-3 / max(1, r["sweep_launches"])
     achieved = bytes_per_launch / avg_sweep_s / 1e9
-    kernel = "k_sweep<%s,%d,%d>" % ("float" if prec == "fp32" else "double", block, ppt)
+    kernel = "k_sweep<%s,%d>" % ("float" if prec == "fp32" else "double", ppt)
     tr = recorded_traffic(prec, kernel, workload_name)
     return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "traffic": (tr["dram_bytes_per_particle"] * launch_ps) if tr else None,
@@ -384,7 +384,7 @@ def run_gpu(args, rank: int, world: int):
         c3 = {"workload": dc.name, "value": r3["ps"] / (r3["total_ms"] * 1e-3), "unit": UNIT,
               "ms_per_step": r3["total_ms"] / 20, "steps": 20, "warmup": 6,
               "particles": int(r3["ps"] / max(1, r3["sweep_launches"])), "clocks": r3["clocks"],
-              "roofline": sweep_roofline(r3, "fp32", args.block, args.ppt, dc.name)}
+              "roofline": sweep_roofline(r3, "fp32", args.ppt, dc.name)}
     rows_f = None
     if not args.quick and not args.no_rows_f:
         # the widened rows on the same workload and launch shape: the leapfrog variant (f2); the
@@ -404,7 +404,7 @@ def run_gpu(args, rank: int, world: int):
         P = d.steps_per_period
         rows_f = {
             "leapfrog": {"value": lf["ps"] / (lf["total_ms"] * 1e-3), "unit": UNIT, "ms_per_step": lf["total_ms"] / n_f,
-                         "roofline": sweep_roofline(lf, "fp32", args.block, args.ppt, d0.name)},
+                         "roofline": sweep_roofline(lf, "fp32", args.ppt, d0.name)},
             "verlet_same_run": {"value": base["ps"] / (base["total_ms"] * 1e-3), "unit": UNIT,
                                 "ms_per_step": base["total_ms"] / n_f},
             "diagnostics_every_step": {
@@ -427,7 +427,7 @@ def run_gpu(args, rank: int, world: int):
     # aggregate over ranks: the job took as long as its slowest rank, and did every rank's work
     total_ms, ps = reduce_over_ranks(main["total_ms"], main["ps"], world, "cuda")
     value = ps / (total_ms * 1e-3)
-    roofline = sweep_roofline(main, "fp32", args.block, args.ppt, d0.name)
+    roofline = sweep_roofline(main, "fp32", args.ppt, d0.name)
 
     res = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
            "warmup": args.warmup, "ms_per_step": total_ms / args.steps, "higher_is_better": True,
@@ -531,7 +531,8 @@ def main():
     ap.add_argument("--warmup", type=int, default=5)
     ap.add_argument("--impl", default="gb300", choices=["gb300", "reference"])
     ap.add_argument("--sort-every", type=int, default=16)
-    ap.add_argument("--block", type=int, default=256)
+    ap.add_argument("--block", type=int, default=256,
+                    help="unit of the library's limit on sweep threads per SM (no effect without such a limit)")
     ap.add_argument("--ppt", type=int, default=4)
     ap.add_argument("--cpu-steps", type=int, default=40)
     ap.add_argument("--no-cpu-baseline", action="store_true")

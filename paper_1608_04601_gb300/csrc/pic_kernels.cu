@@ -265,41 +265,12 @@ __device__ __forceinline__ d4 ldcg_rec(const d4* p) {
     return d4{a.x, a.y, b.x, b.y};
 }
 
-// The random draws, directions and normals of a collision out of line: they appear several times in
-// the sweep, and its instructions are what a short sweep waits for.
-__device__ __forceinline__ U4 draw_call(unsigned long long seed, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3) {
-    return philox4x32_10(c0, c1, c2, c3, (uint32_t)seed, (uint32_t)(seed >> 32));
-}
-__device__ __forceinline__ float3 iso_dir_call(float ua, float ub) {
-    float3 n;
-    iso_dir(ua, ub, n.x, n.y, n.z);
-    return n;
-}
-__device__ __forceinline__ float2 box_muller_call(float ua, float ub) {
-    float2 n;
-    box_muller(ua, ub, n.x, n.y);
-    return n;
-}
-__device__ __forceinline__ void direction(float ua, float ub, float& x, float& y, float& z) {
-    const float3 n = iso_dir_call(ua, ub);
-    x = n.x;
-    y = n.y;
-    z = n.z;
-}
-__device__ __forceinline__ void direction(float ua, float ub, double& x, double& y, double& z) {
-    iso_dir(ua, ub, x, y, z);
-}
-__device__ __forceinline__ void normals(float ua, float ub, float& a, float& b) {
-    const float2 n = box_muller_call(ua, ub);
-    a = n.x;
-    b = n.y;
-}
 // draw() of pic_device.cuh with the counter's second and third words prepared once.
 struct Stream {
     unsigned long long seed;
     uint32_t w1, w2, did;  // step bits 0..31; step bits 32..47 << 16 | species << 8; discharge
     __device__ __forceinline__ U4 draw(uint32_t slot, int call) const {
-        return draw_call(seed, slot, w1, w2 | (uint32_t)call, did);
+        return philox4x32_10(slot, w1, w2 | (uint32_t)call, did, (uint32_t)seed, (uint32_t)(seed >> 32));
     }
 };
 
@@ -352,7 +323,7 @@ __device__ __forceinline__ uint32_t collide(const Seg<T>& S, int SP, unsigned lo
             // the scattered electron's direction: the same draw for every process, so it is
             // formed once, outside the per-process branches
             T nx, ny, nz;
-            direction(u01(r.z), u01(r.w), nx, ny, nz);
+            iso_dir(u01(r.z), u01(r.w), nx, ny, nz);
             if (j == 0) {  // elastic, target at rest: v' = beta v + (1-beta)|v| n
                 const T g = sqrt_(e2);
                 const T og = mul_(K.omb, g);
@@ -380,13 +351,13 @@ __device__ __forceinline__ uint32_t collide(const Seg<T>& S, int SP, unsigned lo
                     vz = mul_(sp, nz);
                     const U4 q1 = rs.draw(slot, 1);
                     const U4 w = rs.draw(slot, 2);
-                    direction(u01(q1.x), u01(q1.y), nx, ny, nz);
+                    iso_dir(u01(q1.x), u01(q1.y), nx, ny, nz);
                     cvx = mul_(sp, nx);
                     cvy = mul_(sp, ny);
                     cvz = mul_(sp, nz);
                     float b0, b1, b2, b3;
-                    normals(u01(q1.z), u01(q1.w), b0, b1);
-                    normals(u01(w.x), u01(w.y), b2, b3);
+                    box_muller(u01(q1.z), u01(q1.w), b0, b1);
+                    box_muller(u01(w.x), u01(w.y), b2, b3);
                     ivx = mul_(K.sig_n, (T)b0);
                     ivy = mul_(K.sig_n, (T)b1);
                     ivz = mul_(K.sig_n, (T)b2);
@@ -423,8 +394,8 @@ __device__ __forceinline__ uint32_t collide(const Seg<T>& S, int SP, unsigned lo
         const U4 r = rs.draw(slot, 0);
         const U4 q1 = rs.draw(slot, 1);
         float a0, a1, a2, a3;
-        normals(u01(q1.x), u01(q1.y), a0, a1);
-        normals(u01(q1.z), u01(q1.w), a2, a3);
+        box_muller(u01(q1.x), u01(q1.y), a0, a1);
+        box_muller(u01(q1.z), u01(q1.w), a2, a3);
         const T vnx = mul_(K.sig_n, (T)a0), vny = mul_(K.sig_n, (T)a1), vnz = mul_(K.sig_n, (T)a2);
         const T gx = sub_(vx, vnx), gy = sub_(vy, vny), gz = sub_(vz, vnz);
         const T g2 = fma_(gx, gx, fma_(gy, gy, mul_(gz, gz)));
@@ -446,7 +417,7 @@ __device__ __forceinline__ uint32_t collide(const Seg<T>& S, int SP, unsigned lo
         if (R < C0) {  // isotropic in the centre-of-mass frame, equal masses
             const T hg = mul_((T)0.5, sqrt_(g2));
             T nx, ny, nz;
-            direction(u01(r.z), u01(r.w), nx, ny, nz);
+            iso_dir(u01(r.z), u01(r.w), nx, ny, nz);
             vx = fma_(hg, nx, mul_(add_(vx, vnx), (T)0.5));
             vy = fma_(hg, ny, mul_(add_(vy, vny), (T)0.5));
             vz = fma_(hg, nz, mul_(add_(vz, vnz), (T)0.5));
@@ -473,7 +444,7 @@ __device__ __forceinline__ bool emit_see(const Seg<T>& S, unsigned long long* Do
     if (!((T)u01(w.x) < K.gamma)) return false;
     const T vn = mul_(K.sig_see_n, (T)__fsqrt_rn(-own_logf(u01(w.y))));
     float t0, t1;
-    normals(u01(w.z), u01(w.w), t0, t1);
+    box_muller(u01(w.z), u01(w.w), t0, t1);
     const int ce = side == 0 ? 0 : S.N - 1;
     const T fe = side == 0 ? (T)0 : one_minus_ulp<T>();
     p = Part<T>{ce, fe, mul_(K.sig_see, (T)t0), mul_(K.sig_see, (T)t1), side == 0 ? vn : -vn};
@@ -2421,9 +2392,10 @@ static cudaError_t smem_attr(K kern, size_t smem) {
 }
 
 // Launch with programmatic stream serialization: the grid may be scheduled while the kernel before
-// it in the stream is still finishing (it takes SMs as they free up), and every such kernel starts
-// with grid_dep_wait(), which returns once that kernel has completed and its memory is visible. So
-// the kernel-to-kernel gap of a step shrinks while the ordering stays that of plain launches.
+// it in the stream is still finishing (it takes SMs as they free up). Every such kernel calls
+// grid_dep_sync() before it touches memory that kernels write, which returns once the kernel before has
+// completed and its writes are visible. So the kernel-to-kernel gap of a step shrinks while the ordering
+// stays that of plain launches.
 template <typename... KArgs, typename... Args>
 static cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                              Args... args) {
