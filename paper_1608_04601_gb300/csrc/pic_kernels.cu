@@ -1963,9 +1963,9 @@ __global__ void __launch_bounds__(DIAG_BLOCK) k_diag(const Disc* __restrict__ di
 // discharges of 2e4 + 2e4 launched 38912 CTAs, most of them empty, in 72 us each. A tile: warp w walks chunks
 // t SORT_NW CPW + w CPW .. + CPW - 1 (CPW = SORT_R 32 / CHUNK) in slot order. What bounds them is latency (of
 // the loads, and of the warp's serial ranks), so many warps with the loads of several rows in flight: 16-bit
-// counters, offsets of 4 rows at a time. Measured on aged stores, the three kernels: 31.5
-// -> 25 us at 2e4 + 2e4 particles (128 cells), 157 -> 67 for 64 such discharges, 40 -> 37 at 1e6 + 1e6
-// (512), 466 -> 366 at 1.2e7 + 1.2e7 (2048). Sorting a store of 2.5e4 whole by one CTA took 40 us.
+// counters, offsets of 4 rows at a time. Measured on aged stores, the three kernels in a row: 33
+// -> 20 us at 2e4 + 2e4 particles (128 cells), 154 -> 51 for 64 such discharges, 45 -> 35 at 1e6 + 1e6
+// (512), 473 -> 298 at 1.2e7 + 1.2e7 (2048). Sorting a store of 2.5e4 whole by one CTA took 40 us.
 __device__ __forceinline__ long long sort_tiles(long long chunks, int chunk) {
     const long long per = (long long)SORT_NW * (SORT_R * 32 / chunk);
     return (chunks + per - 1) / per;
